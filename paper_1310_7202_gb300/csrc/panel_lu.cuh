@@ -20,7 +20,8 @@ struct LuArgs {
   int32_t* psg;        // [C] row at each position < C
   int p0;              // first column of the panel of this launch
   int pw;              // its width
-  int cu;              // the launch solves the pivot rows of columns [p0 + pw, cu) (0: C)
+  int cu;              // the launch solves the pivot rows of columns [p0 + pw, cu) (0: C): the
+  int o0;              //   rows of positions [o0, p0 + pw)
   void* u12;           // [96][ldu] the solved pivot rows of the current panel or block,
   int64_t ldu;         //   dense (row s = pivot p0 + s), read by the trailing update
   void* u12t;          // FP32 only, may be NULL: [2][96][ldu] floats of scratch; when set,
