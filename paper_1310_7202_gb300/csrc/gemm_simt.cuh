@@ -58,6 +58,10 @@ int32_t gemm_simt_batched(const GemmArgs* table_dev, int count, int64_t max_m, i
                           bool a_kmajor, bool b_kmajor, bool c_rowmajor, cudaStream_t s,
                           int tile = 0);
 
+// Slices along K of an FP64 product, for gemm_simt's FP64 tiles: the FP64 units bound it, so
+// that the busiest SM's k-steps count.
+int gemm_splits_f64(int64_t M, int64_t N, int64_t K);
+
 int gemm_tile_m(int32_t dtype);
 int gemm_tile_n(int32_t dtype);
 

@@ -249,14 +249,6 @@ static size_t rs_carve(size_t& cur, size_t bytes) {
   return at;
 }
 
-static int rs_split(int64_t M, int64_t N, int64_t K) {
-  const int bm = gemm_tile_m(RLU_F64), bn = gemm_tile_n(RLU_F64);
-  const int64_t tiles = ceil_div(M, bm) * ceil_div(N, bn);
-  int64_t s = ceil_div(2 * (int64_t)sm_count(), tiles);
-  const int64_t kmax = K / 64 > 1 ? K / 64 : 1;
-  return (int)(s < 1 ? 1 : (s > kmax ? kmax : s));
-}
-
 static bool rsvd_plan(int64_t m, int64_t n, int k, int l, RsvdPlan& p) {
   if (!(k >= 1 && k <= l && l <= m && l <= n) || l > 4096) return false;
   if (m > INT32_MAX / 2 || n > INT32_MAX / 2) return false;
@@ -266,10 +258,10 @@ static bool rsvd_plan(int64_t m, int64_t n, int k, int l, RsvdPlan& p) {
   p.ldg = round_up(n, 8);
   p.ldy = round_up(m, 8);
   p.ldw = l;
-  p.split_y = rs_split(m, l, n);
-  p.split_g = rs_split(l, l, m);
-  p.split_q = rs_split(m, k, l);
-  p.split_b = rs_split(k, n, m);
+  p.split_y = gemm_splits_f64(m, l, n);
+  p.split_g = gemm_splits_f64(l, l, m);
+  p.split_q = gemm_splits_f64(m, k, l);
+  p.split_b = gemm_splits_f64(k, n, m);
   size_t part = 0;
   auto upd = [&](size_t b) { part = b > part ? b : part; };
   upd(gemm_partial_bytes<double>(m, l, p.split_y));
