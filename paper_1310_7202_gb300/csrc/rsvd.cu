@@ -12,7 +12,8 @@
 //   and B = Q^T A, so that Q B = Q Q^T A is the rank-k approximation whose error
 //   ||Q Q^T A - A|| Section 5 compares with the randomized LU's.
 //
-// The Jacobi eigensolver (parallel two-sided Jacobi): the l x l matrix (l rounded up to an
+// The Jacobi eigensolver (parallel two-sided Jacobi; k_jacobi_smem for l <= 112, k_jacobi_sym
+// above): the l x l matrix (l rounded up to an
 // even l2; a padding index stays decoupled) is swept by the round-robin (circle) schedule:
 // each round pairs every index with one other, and the l2 / 2 rotations of a round commute,
 // so M <- J^T M J updates every 2 x 2 block (pair i, pair j) independently from the old
@@ -181,6 +182,154 @@ __global__ void __launch_bounds__(JAC_T) k_jacobi_sym(JacArgs a) {
   }
 }
 
+// The same sweeps for l2 <= JAC_SMEM_MAX in one CTA with M and V in shared memory, updated in
+// place (a 2 x 2 block of M is read and written by one thread). What bounds a round is the
+// chain of a rotation (two reciprocal square roots) and the SM's FP64 units (2 multiply-adds a
+// cycle), so M's symmetric half is computed once and mirrored, and V takes a round's rotations
+// while the next round's are computed. A round with the matrices in global memory and IEEE
+// divisions and square roots took 9.4 us at l2 = 44.
+//
+// With d = m_qq - m_pp, b = 2 m_pq and h = sqrt(d^2 + b^2), the smaller rotation that zeroes
+// m_pq has cos 2phi = |d| / h: c = sqrt((1 + |d| / h) / 2), s = sign(d) b / (2 h c).
+static constexpr int JAC_SMEM_MAX = 112;
+static constexpr int JAC_ST = 512;
+
+static size_t jac_smem_bytes(int l2) {
+  const int P = l2 / 2;
+  return sizeof(double) * 2 * (size_t)l2 * (l2 | 1) + 2 * (size_t)P * (sizeof(double2) + sizeof(int2)) +
+         sizeof(ushort2) * (size_t)(P * (P + 1) / 2);
+}
+
+__global__ void __launch_bounds__(JAC_ST) k_jacobi_smem(JacArgs a) {
+  extern __shared__ __align__(16) unsigned char jac_smem[];
+  const int l2 = a.l2, P = l2 / 2, ld = l2 | 1, tid = threadIdx.x, n1 = l2 - 1;
+  double* M = reinterpret_cast<double*>(jac_smem);     // row-major
+  double* V = M + (size_t)l2 * ld;                     // column-major
+  double2* cs = reinterpret_cast<double2*>(jac_smem + (2 * sizeof(double) * l2 * ld + 15) / 16 * 16);
+  int2* pq = reinterpret_cast<int2*>(cs + 2 * P);      // [2][P] each, by the round's parity
+  ushort2* ij = reinterpret_cast<ushort2*>(pq + 2 * P);  // block pairs i <= j
+  __shared__ int s_cnt[2];                             // rotations, by the sweep's parity
+  for (int e = tid; e < l2 * l2; e += JAC_ST) {
+    M[e / l2 * ld + e % l2] = a.M0[e];
+    V[e / l2 * ld + e % l2] = a.V0[e];
+  }
+  for (int j = tid; j < P; j += JAC_ST)
+    for (int i = 0; i <= j; ++i)
+      ij[j * (j + 1) / 2 + i] = make_ushort2((unsigned short)i, (unsigned short)j);
+  if (tid < 2) s_cnt[tid] = 0;
+  __syncthreads();
+  const int RW = (P + 31) / 32 * 32;  // threads that compute rotations
+  auto turn_v = [&](int par, int t0, int nt) {  // V' = V J of one round
+    const double2* c2 = cs + par * P;
+    const int2* p2 = pq + par * P;
+    for (int it = t0; it < P * l2; it += nt) {
+      const int j = it / l2, row = it - j * l2;
+      const double2 r = c2[j];
+      if (r.y == 0.0) continue;
+      double* vp = V + p2[j].x * ld + row;
+      double* vq = V + p2[j].y * ld + row;
+      const double x = *vp, y = *vq;
+      *vp = r.x * x - r.y * y;
+      *vq = r.y * x + r.x * y;
+    }
+  };
+  int sweep = 0, round = 0;
+  for (; sweep < JAC_MAX_SWEEPS; ++sweep) {
+    for (int r = 0; r < n1; ++r, ++round) {
+      const int par = round & 1;
+      if (tid < RW) {
+        if (tid < P) {
+          const int i = tid;
+          int x, y;
+          if (i == 0) {
+            x = 0;
+            y = 1 + r;
+          } else {
+            x = i + r;
+            y = n1 - i + r;
+            x = 1 + (x >= n1 ? x - n1 : x);
+            y = 1 + (y >= n1 ? y - n1 : y);
+          }
+          const int p = min(x, y), q = max(x, y);
+          const double app = M[p * ld + p], aqq = M[q * ld + q], apq = M[p * ld + q];
+          double c = 1.0, s = 0.0;
+          const double d = aqq - app, b = 2.0 * apq;
+          const double big = fmax(fmax(fabs(app), fabs(aqq)), fabs(apq));
+          const bool sq = big > 1e-130 && big < 1e140;  // squares stay in range
+          if (sq ? apq * apq > 1e-30 * fabs(app) * fabs(aqq)
+                 : fabs(apq) > 1e-15 * sqrt(fabs(app) * fabs(aqq)) && apq != 0.0) {
+            if (sq) {
+              const double ih = rsqrt(fma(d, d, b * b));
+              const double c2 = fma(0.5 * fabs(d), ih, 0.5);
+              const double ic = rsqrt(c2);
+              c = c2 * ic;
+              s = 0.5 * (d >= 0 ? b : -b) * ih * ic;
+            } else {
+              const double theta = d / b;
+              const double t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
+              c = 1.0 / sqrt(t * t + 1.0);
+              s = t * c;
+            }
+            if (s != 0.0) atomicAdd(&s_cnt[sweep & 1], 1);
+          }
+          cs[par * P + i] = make_double2(c, s);
+          pq[par * P + i] = make_int2(p, q);
+        }
+      } else if (round > 0) {
+        turn_v(par ^ 1, tid - RW, JAC_ST - RW);
+      }
+      __syncthreads();
+      // M' = J^T M J, block (pair i, pair j) and its mirror image
+      for (int it = tid; it < P * (P + 1) / 2; it += JAC_ST) {
+        const int i = ij[it].x, j = ij[it].y;
+        const double2 ri = cs[par * P + i], rj = cs[par * P + j];
+        if (ri.y == 0.0 && rj.y == 0.0) continue;
+        const int2 ki = pq[par * P + i], kj = pq[par * P + j];
+        double* m0 = M + ki.x * ld;
+        double* m1 = M + ki.y * ld;
+        const double x00 = m0[kj.x], x01 = m0[kj.y], x10 = m1[kj.x], x11 = m1[kj.y];
+        // columns: p <- c x_p - s x_q, q <- s x_p + c x_q; then rows, the rotation of pair i
+        const double y00 = rj.x * x00 - rj.y * x01, y01 = rj.y * x00 + rj.x * x01;
+        const double y10 = rj.x * x10 - rj.y * x11, y11 = rj.y * x10 + rj.x * x11;
+        const double z00 = ri.x * y00 - ri.y * y10, z11 = ri.y * y01 + ri.x * y11;
+        double z10 = ri.y * y00 + ri.x * y10, z01 = ri.x * y01 - ri.y * y11;
+        if (i == j) {  // the annihilated pair
+          z01 = 0.0;
+          z10 = 0.0;
+        }
+        m0[kj.x] = z00;
+        m0[kj.y] = z01;
+        m1[kj.x] = z10;
+        m1[kj.y] = z11;
+        if (i != j) {
+          M[kj.x * ld + ki.x] = z00;
+          M[kj.y * ld + ki.x] = z01;
+          M[kj.x * ld + ki.y] = z10;
+          M[kj.y * ld + ki.y] = z11;
+        }
+      }
+      __syncthreads();
+    }
+    const int turned = s_cnt[sweep & 1];
+    if (tid == 0) s_cnt[(sweep + 1) & 1] = 0;
+    __syncthreads();
+    if (turned == 0) {
+      ++sweep;
+      break;
+    }
+  }
+  turn_v((round - 1) & 1, tid, JAC_ST);
+  __syncthreads();
+  for (int e = tid; e < l2 * l2; e += JAC_ST) {
+    a.M0[e] = M[e / l2 * ld + e % l2];
+    a.V0[e] = V[e / l2 * ld + e % l2];
+  }
+  if (tid == 0) {
+    a.result[0] = 0;
+    a.result[1] = sweep;
+  }
+}
+
 // M (l x l FP64, row-major, ld l2) padded to l2 with a decoupled unit entry; V = I (l2 x l2).
 __global__ void k_jacobi_init(double* M, double* V, int l, int l2) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)l2 * l2;
@@ -338,7 +487,13 @@ extern "C" int32_t rlu_rsvd(const void* A, int32_t dtype, int64_t m, int64_t n, 
   ja.nrot = hdr + 32;
   ja.result = reinterpret_cast<int*>(hdr + 96);
   ja.status = status;
-  {
+  if (l2 <= JAC_SMEM_MAX) {
+    const size_t smem = jac_smem_bytes(l2);
+    RLU_CUDA_TRY(cudaFuncSetAttribute(k_jacobi_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)smem));
+    k_jacobi_smem<<<1, JAC_ST, smem, s>>>(ja);
+    RLU_TRY(last_launch_status());
+  } else {
     const int P = l2 / 2;
     const size_t smem = (size_t)P * (sizeof(double2) + sizeof(int2));
     const void* fn = reinterpret_cast<const void*>(&k_jacobi_sym);
