@@ -1,0 +1,54 @@
+"""||PAQ - LU|| in its exact-FP32 and FP64 forms: odd sizes, operands outside the FP32 form's
+range, and values that no comparison with a range accepts."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1310_7202_gb300 import rlu
+
+pytestmark = pytest.mark.gpu
+
+
+def case(m, n, k, dtype, scale, seed):
+    rng = np.random.default_rng(seed)
+    L = rng.standard_normal((m, k)).astype(np.float32)
+    U = (rng.standard_normal((k, n)) * scale).astype(np.float32)
+    A = (L.astype(np.float64) @ U.astype(np.float64)
+         + 1e-3 * scale * rng.standard_normal((m, n))).astype(np.float32)
+    At = torch.from_numpy(A).cuda().to(dtype)
+    P, Q = rng.permutation(m).astype(np.int32), rng.permutation(n).astype(np.int32)
+    Lt = torch.from_numpy(np.ascontiguousarray(L.T)).cuda().t()
+    args = (At, torch.from_numpy(P).cuda(), torch.from_numpy(Q).cuda(), Lt, torch.from_numpy(U).cuda())
+    R = At.double().cpu().numpy()[P][:, Q] - L.astype(np.float64) @ U.astype(np.float64)
+    return args, R
+
+
+# the FP32 form drops nothing above 2^-70 of a term; FP64 rounds k additions at 2^-53 of terms
+# of order 4 sqrt(k) scale in residuals of order 1e-3 scale or more
+@pytest.mark.parametrize("m,n,k,dtype,scale", [
+    (1, 1, 1, torch.float32, 1.0), (65, 63, 17, torch.float32, 1.0), (513, 1030, 33, torch.float32, 1.0),
+    (5003, 131, 16, torch.float32, 2.0 ** -10), (300, 257, 40, torch.bfloat16, 1.0),
+    (200, 190, 20, torch.float32, 2.0 ** 60), (200, 190, 20, torch.float32, 2.0 ** -60)])
+def test_norms(m, n, k, dtype, scale):
+    args, R = case(m, n, k, dtype, scale, m + n)
+    fro, spec = rlu.reconstruct_error(*args, power_iters=300)
+    want = np.linalg.norm(R)
+    assert abs(float(fro) - want) <= 1e-12 * want
+    top = np.linalg.norm(R, 2)
+    assert float(spec) <= top * (1 + 1e-12) and float(spec) >= 0.97 * top
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_nonfinite_reaches_the_result(bad):
+    args, _ = case(130, 70, 9, torch.float32, 1.0, 5)
+    args[0][17, 33] = bad
+    fro, _ = rlu.reconstruct_error(*args, power_iters=2)
+    assert not np.isfinite(float(fro))
+
+
+def test_zero():
+    args, _ = case(40, 50, 3, torch.float32, 1.0, 6)
+    for t in (args[0], args[3], args[4]):
+        t.zero_()
+    fro, spec = rlu.reconstruct_error(*args, power_iters=3)
+    assert float(fro) == 0.0 and float(spec) == 0.0
