@@ -189,57 +189,101 @@ __global__ void k_philox_u32(uint64_t seed, uint32_t stream_id, uint64_t first,
   }
 }
 
+// Column j and row i of element e of an n-row G, by a 32-bit division where e < total fits (the
+// 64-bit ones of every element took longer than the rest of the FP32 kernel: 8192 x 210 in
+// 10 us).
+__device__ __forceinline__ void locate(int64_t e, int64_t n, int64_t total, int64_t& j, int64_t& i) {
+  if (total <= 0xffffffffll) {
+    const uint32_t q = (uint32_t)e / (uint32_t)n;
+    j = q;
+    i = (uint32_t)e - q * (uint32_t)n;
+  } else {
+    j = e / n;
+    i = e - j * n;
+  }
+}
+__device__ __forceinline__ void put4(float* p, const float (&z)[4]) {
+  *reinterpret_cast<float4*>(p) = make_float4(z[0], z[1], z[2], z[3]);
+}
+__device__ __forceinline__ void put4(__nv_bfloat16* p, const float (&z)[4]) {
+  __nv_bfloat162 v[2];
+  v[0] = __nv_bfloat162(__float2bfloat16_rn(z[0]), __float2bfloat16_rn(z[1]));
+  v[1] = __nv_bfloat162(__float2bfloat16_rn(z[2]), __float2bfloat16_rn(z[3]));
+  *reinterpret_cast<uint2*>(p) = *reinterpret_cast<const uint2*>(v);
+}
+__device__ __forceinline__ void put1(float* p, float z) { *p = z; }
+__device__ __forceinline__ void put1(__nv_bfloat16* p, float z) { *p = __float2bfloat16_rn(z); }
+
+// The four deviates of counter c; vec: n and ldg are multiples of 4 and G is aligned to four
+// elements, so that they lie in one column and one aligned piece.
 template <typename OutT>
-__device__ __forceinline__ void store_g(OutT* G, int64_t ldg, int64_t n, int64_t e, float v);
-
-template <>
-__device__ __forceinline__ void store_g<float>(float* G, int64_t ldg, int64_t n, int64_t e,
-                                               float v) {
-  G[(e / n) * ldg + (e % n)] = v;
+__device__ __forceinline__ void gauss32_counter(int64_t c, uint32_t k0, uint32_t k1,
+                                                uint32_t stream_id, int64_t n, int64_t total,
+                                                OutT* G, int64_t ldg, bool vec,
+                                                const SeriesCoefs& C) {
+  const uint4 w = philox10(make_uint4((uint32_t)c, (uint32_t)((uint64_t)c >> 32), stream_id, 0u),
+                           k0, k1);
+  float z[4];
+  box_muller32(w.x, w.y, C, z[0], z[1]);
+  box_muller32(w.z, w.w, C, z[2], z[3]);
+  int64_t j, i;
+  locate(4 * c, n, total, j, i);
+  if (vec) {
+    put4(G + j * ldg + i, z);
+    return;
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    if (4 * c + t < total) put1(G + j * ldg + i, z[t]);
+    if (++i == n) {
+      i = 0;
+      ++j;
+    }
+  }
 }
-template <>
-__device__ __forceinline__ void store_g<__nv_bfloat16>(__nv_bfloat16* G, int64_t ldg,
-                                                       int64_t n, int64_t e, float v) {
-  G[(e / n) * ldg + (e % n)] = __float2bfloat16_rn(v);
+
+// Sets info to "no error" (the first kernel of a factorization does it for the rest).
+__device__ __forceinline__ void reset_info(rlu_info* info) {
+  if (info && blockIdx.x == 0 && threadIdx.x == 0) *info = rlu_info{RLU_OK, -1, -1, 0};
 }
 
-__global__ void k_gauss64(uint64_t seed, uint32_t stream_id, int64_t n, int64_t total,
-                          double* __restrict__ G, int64_t ldg, SeriesCoefs C) {
+// FP64: a thread takes one pair of a counter's four deviates, in blocks of one warp, so that
+// the ~200 FP64 operations of a pair reach every SM's FP64 units also for a small G (512 x 25:
+// 19 us with a counter per thread in 13 blocks).
+__global__ void __launch_bounds__(32) k_gauss64(uint64_t seed, uint32_t stream_id, int64_t n,
+                                                int64_t total, double* __restrict__ G,
+                                                int64_t ldg, SeriesCoefs C, rlu_info* info) {
+  reset_info(info);
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-  const int64_t nc = (total + 3) / 4;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc;
-       c += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t np = (total + 1) / 2;
+  for (int64_t p = blockIdx.x * 32ll + threadIdx.x; p < np; p += gridDim.x * 32ll) {
+    const int64_t c = p >> 1;
     const uint4 w = philox10(make_uint4((uint32_t)c, (uint32_t)((uint64_t)c >> 32), stream_id,
                                         0u), k0, k1);
-    double z[4];
-    box_muller64(w.x, w.y, C, z[0], z[1]);
-    box_muller64(w.z, w.w, C, z[2], z[3]);
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int64_t e = 4 * c + t;
-      if (e < total) G[(e / n) * ldg + (e % n)] = z[t];
+    const bool second = p & 1;
+    double z0, z1;
+    box_muller64(second ? w.z : w.x, second ? w.w : w.y, C, z0, z1);
+    int64_t j, i;
+    locate(2 * p, n, total, j, i);
+    G[j * ldg + i] = z0;
+    if (++i == n) {
+      i = 0;
+      ++j;
     }
+    if (2 * p + 1 < total) G[j * ldg + i] = z1;
   }
 }
 
 template <typename OutT>
 __global__ void k_gauss32(uint64_t seed, uint32_t stream_id, int64_t n, int64_t total,
-                          OutT* __restrict__ G, int64_t ldg, SeriesCoefs C) {
+                          OutT* __restrict__ G, int64_t ldg, bool vec, SeriesCoefs C,
+                          rlu_info* info) {
+  reset_info(info);
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
   const int64_t nc = (total + 3) / 4;
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc;
-       c += (int64_t)gridDim.x * blockDim.x) {
-    const uint4 w = philox10(make_uint4((uint32_t)c, (uint32_t)((uint64_t)c >> 32), stream_id,
-                                        0u), k0, k1);
-    float z[4];
-    box_muller32(w.x, w.y, C, z[0], z[1]);
-    box_muller32(w.z, w.w, C, z[2], z[3]);
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int64_t e = 4 * c + t;
-      if (e < total) store_g<OutT>(G, ldg, n, e, z[t]);
-    }
-  }
+       c += (int64_t)gridDim.x * blockDim.x)
+    gauss32_counter(c, k0, k1, stream_id, n, total, G, ldg, vec, C);
 }
 
 // Batched FP32 G: problem blockIdx.y of the table, its own seed and sizes.
@@ -247,19 +291,10 @@ __global__ void k_gauss32_batched(const GaussJob* __restrict__ jobs, SeriesCoefs
   const GaussJob j = jobs[blockIdx.y];
   const uint32_t k0 = (uint32_t)j.seed, k1 = (uint32_t)(j.seed >> 32);
   const int64_t total = j.n * j.l, nc = (total + 3) / 4;
+  const bool vec = j.n % 4 == 0 && j.ldg % 4 == 0 && ((uintptr_t)j.G & 15u) == 0;
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc;
-       c += (int64_t)gridDim.x * blockDim.x) {
-    const uint4 w = philox10(make_uint4((uint32_t)c, (uint32_t)((uint64_t)c >> 32), 0u, 0u), k0,
-                             k1);
-    float z[4];
-    box_muller32(w.x, w.y, C, z[0], z[1]);
-    box_muller32(w.z, w.w, C, z[2], z[3]);
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int64_t e = 4 * c + t;
-      if (e < total) j.G[(e / j.n) * j.ldg + (e % j.n)] = z[t];
-    }
-  }
+       c += (int64_t)gridDim.x * blockDim.x)
+    gauss32_counter(c, k0, k1, 0u, j.n, total, j.G, j.ldg, vec, C);
 }
 
 int32_t launch_gaussian_batched(const GaussJob* jobs_dev, int count, cudaStream_t s) {
@@ -277,19 +312,24 @@ static int grid_for(int64_t work, int threads) {
 }
 
 int32_t launch_gaussian(uint64_t seed, uint32_t stream_id, int64_t n, int64_t l, int32_t dtype,
-                        void* G, int64_t ldg, cudaStream_t s) {
+                        void* G, int64_t ldg, cudaStream_t s, rlu_info* info) {
   const int64_t total = n * l;
   if (total == 0) return RLU_OK;
   static const SeriesCoefs C = make_coefs();
   const int threads = 256;
   const int grid = grid_for(ceil_div(total, 4), threads);
+  auto vec = [&](int size) {
+    return n % 4 == 0 && ldg % 4 == 0 && ((uintptr_t)G & (4 * size - 1u)) == 0;
+  };
   if (dtype == RLU_F64) {
-    k_gauss64<<<grid, threads, 0, s>>>(seed, stream_id, n, total, (double*)G, ldg, C);
+    k_gauss64<<<8 * grid_for(ceil_div(total, 2), threads), 32, 0, s>>>(seed, stream_id, n, total,
+                                                                     (double*)G, ldg, C, info);
   } else if (dtype == RLU_F32) {
-    k_gauss32<float><<<grid, threads, 0, s>>>(seed, stream_id, n, total, (float*)G, ldg, C);
+    k_gauss32<float><<<grid, threads, 0, s>>>(seed, stream_id, n, total, (float*)G, ldg, vec(4), C,
+                                              info);
   } else if (dtype == RLU_BF16) {
     k_gauss32<__nv_bfloat16><<<grid, threads, 0, s>>>(seed, stream_id, n, total,
-                                                      (__nv_bfloat16*)G, ldg, C);
+                                                      (__nv_bfloat16*)G, ldg, vec(2), C, info);
   } else {
     return RLU_EUNSUPPORTED;
   }
@@ -315,5 +355,5 @@ extern "C" int32_t rlu_philox_u32(uint64_t seed, uint32_t stream_id, uint64_t fi
 extern "C" int32_t rlu_gaussian(uint64_t seed, uint32_t stream_id, int64_t n, int64_t l,
                                 int32_t dtype, void* G, int64_t ldg, void* stream) {
   if (G == nullptr || n < 0 || l < 0 || ldg < n || ldg < 1) return RLU_EINVAL;
-  return rlu::launch_gaussian(seed, stream_id, n, l, dtype, G, ldg, (cudaStream_t)stream);
+  return rlu::launch_gaussian(seed, stream_id, n, l, dtype, G, ldg, (cudaStream_t)stream, nullptr);
 }

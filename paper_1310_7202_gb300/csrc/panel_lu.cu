@@ -275,7 +275,10 @@ __global__ void __launch_bounds__(LU_NT, 1) k_cluster_lu(LuArgs a) {
     cl.sync();
   }
 
-  for (int t = tid; t < nr; t += LU_NT) a.perm[posl[t]] = r0 + t;
+  for (int t = tid; t < nr; t += LU_NT) {
+    a.perm[posl[t]] = r0 + t;
+    if (a.posg) a.posg[r0 + t] = posl[t];
+  }
   if (tid == 0) {
     if (crank == 0 && a.zero_step && first_zero >= 0) atomicCAS(a.zero_step, -1, first_zero);
     if (s_nonfinite && a.nonfinite) atomicOr(a.nonfinite, 1);

@@ -15,8 +15,9 @@ struct LuArgs {
   int32_t* zero_step;  // out: first step with a zero pivot, -1 if none (may be NULL)
   int32_t* nonfinite;  // out: OR-ed with 1 when a NaN/Inf is met (may be NULL)
   int32_t* status;     // out: set to RLU_ETIMEOUT if a cluster wait gave up (may be NULL)
-  // register kernel only: position state kept between its per-panel launches
-  int32_t* posg;       // [R] current position of every row
+  int32_t* posg;       // [R] out: position of every row (the register kernel also keeps it here
+                       //   between its per-panel launches; NULL: not written)
+  // register kernel only
   int32_t* psg;        // [C] row at each position < C
   int p0;              // first column of the panel of this launch
   int pw;              // its width

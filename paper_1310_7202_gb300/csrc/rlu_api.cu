@@ -25,7 +25,7 @@
 namespace rlu {
 
 int32_t launch_gaussian(uint64_t seed, uint32_t stream_id, int64_t n, int64_t l, int32_t dtype,
-                        void* G, int64_t ldg, cudaStream_t s);
+                        void* G, int64_t ldg, cudaStream_t s, rlu_info* info);
 
 static std::atomic<uint64_t> g_launches{0};
 void note_launches(int count) { g_launches.fetch_add((uint64_t)count, std::memory_order_relaxed); }
@@ -282,10 +282,9 @@ static int32_t factor_t(const Plan& p, const void* Av, int64_t lda, uint64_t see
   const int k = p.k, l = p.l;
 
   const StepTimer tm{st};
-  if (info) RLU_TRY(info_init(info, s));
-  // step 1
+  // step 1 (its kernel also resets info)
   RLU_TRY(tm.rec(0, false, s));
-  RLU_TRY(launch_gaussian(seed, 0, n, l, (bf16 && !fp8) ? RLU_BF16 : p.dt, G, p.ldg, s));
+  RLU_TRY(launch_gaussian(seed, 0, n, l, (bf16 && !fp8) ? RLU_BF16 : p.dt, G, p.ldg, s, info));
   if (fp8)  // e4m3 G with one scale per 128 x 128 block
     RLU_TRY(fp8_quantize_g(reinterpret_cast<const float*>(G), p.ldg, n, l,
                            reinterpret_cast<uint8_t*>(ws + p.off_G8), p.ld8,
@@ -380,7 +379,7 @@ static int32_t factor_t(const Plan& p, const void* Av, int64_t lda, uint64_t see
     a.ldu = p.ldu12;
     a.u12t = p.off_u12t ? ws + p.off_u12t : nullptr;
     RLU_TRY(launch_cluster_lu(p.dt, false, a, s));
-    return build_ly<T>(X, ld, rows, l, perm, Ln, nullptr, ld, s, hi, lo, parts);
+    return build_ly<T>(X, ld, rows, l, a.posg, Ln, nullptr, ld, s, hi, lo, parts);
   };
   for (int it = 0; it < p.q; ++it) {
     T* Z = reinterpret_cast<T*>(ws + p.off_Z);  // n x l, column-major, ld ldg
@@ -527,7 +526,10 @@ static int32_t factor_t(const Plan& p, const void* Av, int64_t lda, uint64_t see
     bp.mid = reinterpret_cast<__nv_bfloat16*>(ws + p.off_Bm);
     bp.lo = reinterpret_cast<__nv_bfloat16*>(ws + p.off_Bl);
   }
-  RLU_TRY(build_ly<T>(Y, p.ldy, m, k, P, Lt, Lp, p.ldl, s, Lhi, Llo, bp));
+  // L~ itself is read by the SIMT products only
+  const bool simt_c = !(bf16 || (Lhi && tma_ok));
+  RLU_TRY(build_ly<T>(Y, p.ldy, m, k, reinterpret_cast<const int32_t*>(ws + p.off_pos),
+                      simt_c || !Lhi ? Lt : nullptr, Lp, p.ldl, s, Lhi, Llo, bp));
   RLU_TRY(tm.rec(3, true, s));
   if (st && st->Ly) RLU_TRY(copy_cm<T>(Lp, p.ldl, static_cast<T*>(st->Ly), m, m, k, s));
   // step 5: Gram M = L~^T L~ in FP64
@@ -612,7 +614,9 @@ static int32_t factor_t(const Plan& p, const void* Av, int64_t lda, uint64_t see
   }
   // B = M^{-1} C = L^{-T} D^{-1} L^{-1} C
   RLU_TRY(tm.rec(7, false, s));
-  RLU_TRY(trsm_ldl<T>(ldl, Cb, p.ldb, n, Bb, p.ldb, s));
+  // FP64: 32 columns a CTA where 64 would leave SMs' FP64 units idle (and the narrow form fits)
+  RLU_TRY(trsm_ldl<T>(ldl, Cb, p.ldb, n, Bb, p.ldb, s,
+                      sizeof(T) == 8 && ceil_div(n, 64) < sm_count() && k <= 256));
   RLU_TRY(tm.rec(7, true, s));
   if (st && st->B) RLU_TRY(copy_cm<T>(Bb, p.ldb, static_cast<T*>(st->B), n, n, k, s));
   // step 6: LU of B^T (n x k, col-major = B row-major), Crout form
@@ -633,22 +637,21 @@ static int32_t factor_t(const Plan& p, const void* Av, int64_t lda, uint64_t see
   RLU_TRY(tm.rec(8, true, s));
   // step 8 (and L_b for step 7)
   RLU_TRY(tm.rec(9, false, s));
-  RLU_TRY(gather_lb_u<T>(Bb, p.ldb, Q, k, n, Lb, U, ldu, s));
+  // (with L_b's TF32 split where step 7 runs on the tensor cores)
+  const int64_t kb = round_up(k, 4);
+  T* Lbh = p.off_Lbh ? reinterpret_cast<T*>(ws + p.off_Lbh) : nullptr;
+  T* Lbl = p.off_Lbh ? reinterpret_cast<T*>(ws + p.off_Lbl) : nullptr;
+  RLU_TRY(gather_lb_u<T>(Bb, p.ldb, Q, k, n, Lbh ? nullptr : Lb, Lbh, Lbl, kb, U, ldu, s));
   RLU_TRY(tm.rec(9, true, s));
   // step 7: L = L_y L_b
   RLU_TRY(tm.rec(10, false, s));
-  if (p.off_Lbh) {  // three TF32 products: L_y (column-major, i.e. K x M row-major) is
+  if (Lbh) {  // three TF32 products: L_y (column-major, i.e. K x M row-major) is
                     // transposed and split on chip as in the C product; L_b pre-split
-    float* Lbh = reinterpret_cast<float*>(ws + p.off_Lbh);
-    float* Lbl = reinterpret_cast<float*>(ws + p.off_Lbl);
-    const int64_t kb = round_up(k, 4);
-    RLU_TRY(split_parts(reinterpret_cast<const float*>(Lb), k, k, k, Lbh, Lbl, Bf16Parts{}, s,
-                        kb));
     Umma3Op op{};
     op.A0 = reinterpret_cast<const float*>(Lp);
     op.lda = p.ldl;
-    op.B0 = Lbh;
-    op.B1 = Lbl;
+    op.B0 = reinterpret_cast<const float*>(Lbh);
+    op.B1 = reinterpret_cast<const float*>(Lbl);
     op.ldb = kb;
     op.M = m;
     op.N = k;

@@ -30,7 +30,7 @@
 namespace rlu {
 
 int32_t launch_gaussian(uint64_t seed, uint32_t stream_id, int64_t n, int64_t l, int32_t dtype,
-                        void* G, int64_t ldg, cudaStream_t s);
+                        void* G, int64_t ldg, cudaStream_t s, rlu_info* info);
 
 static constexpr int JAC_T = 256;
 static constexpr int JAC_MAX_SWEEPS = 30;
@@ -461,9 +461,8 @@ extern "C" int32_t rlu_rsvd(const void* A, int32_t dtype, int64_t m, int64_t n, 
   const double* Ad = static_cast<const double*>(A);
   const int l2 = p.l2;
   int32_t* status = info ? &info->status : nullptr;
-  if (info) RLU_TRY(info_init(info, s));
-  // steps 1-2
-  RLU_TRY(launch_gaussian(seed, 0, n, l, RLU_F64, G, p.ldg, s));
+  // steps 1-2 (the first kernel also resets info)
+  RLU_TRY(launch_gaussian(seed, 0, n, l, RLU_F64, G, p.ldg, s, info));
   {
     GemmOp op{Ad, lda, true, G, p.ldg, true, Y, p.ldy, false, m, l, n, p.split_y, part, false};
     RLU_TRY((gemm_simt<double, double>(op, s)));

@@ -44,20 +44,65 @@ __device__ __forceinline__ void bf16_split3(float x, __nv_bfloat16* h, __nv_bflo
   lo[at] = __float2bfloat16_rn(r2);
 }
 
+// Column c of L~ and its splits by the row, four rows a thread: Y is read and L~ and its parts
+// written along columns, and only Lp, in pivot order, is scattered (by the pivot position, Y
+// and all seven outputs but Lp were: 131 us at 32768 x 512 with the BF16 parts). vec: bases and
+// leading dimensions suit four elements.
 template <typename T>
-__global__ void k_build_ly(const T* __restrict__ Y, int64_t ldy, int64_t m, int k,
-                           const int32_t* __restrict__ perm, T* __restrict__ Lt,
-                           T* __restrict__ Lp, int64_t ldl, T* __restrict__ Lhi,
-                           T* __restrict__ Llo, Bf16Parts bp) {
+__global__ void __launch_bounds__(256) k_build_ly(const T* __restrict__ Y, int64_t ldy, int64_t m,
+                                                  const int32_t* __restrict__ pos,
+                                                  T* __restrict__ Lt, T* __restrict__ Lp,
+                                                  int64_t ldl, T* __restrict__ Lhi,
+                                                  T* __restrict__ Llo, Bf16Parts bp, bool vec) {
   const int c = blockIdx.y;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < m;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = perm[p];
-    const T v = (c < p) ? Y[(int64_t)c * ldy + r] : (c == p ? T(1) : T(0));
-    if (Lp) Lp[(int64_t)c * ldl + p] = v;
-    if (Lt) Lt[(int64_t)c * ldl + r] = v;
-    if (Lhi) tf32_split(v, Lhi, Llo, (int64_t)c * ldl + r);
-    if (bp.hi) bf16_split3((float)v, bp.hi, bp.mid, bp.lo, (int64_t)c * ldl + r);
+  const int64_t r0 = (blockIdx.x * 256ll + threadIdx.x) * 4;
+  if (r0 >= m) return;
+  const int rows = (int)(m - r0 < 4 ? m - r0 : 4);
+  const int64_t at = (int64_t)c * ldl + r0;
+  struct alignas(4 * sizeof(T)) V4 { T v[4]; };
+  struct alignas(8) B4 { __nv_bfloat16 v[4]; };
+  V4 x, h, l;
+  if (vec && rows == 4) {
+    x = *reinterpret_cast<const V4*>(Y + (int64_t)c * ldy + r0);
+  } else {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x.v[u] = u < rows ? Y[(int64_t)c * ldy + r0 + u] : T(0);
+  }
+  B4 b0, b1, b2;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int p = u < rows ? pos[r0 + u] : -1;
+    x.v[u] = c < p ? x.v[u] : (c == p ? T(1) : T(0));
+    if (Lp && p >= 0 && p < m) Lp[(int64_t)c * ldl + p] = x.v[u];
+    if (Lhi) tf32_split(x.v[u], h.v, l.v, u);
+    if (bp.hi) bf16_split3((float)x.v[u], b0.v, b1.v, b2.v, u);
+  }
+  if (vec && rows == 4) {
+    if (Lt) *reinterpret_cast<V4*>(Lt + at) = x;
+    if (Lhi) {
+      *reinterpret_cast<V4*>(Lhi + at) = h;
+      *reinterpret_cast<V4*>(Llo + at) = l;
+    }
+    if (bp.hi) {
+      *reinterpret_cast<B4*>(bp.hi + at) = b0;
+      *reinterpret_cast<B4*>(bp.mid + at) = b1;
+      *reinterpret_cast<B4*>(bp.lo + at) = b2;
+    }
+    return;
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    if (u >= rows) break;
+    if (Lt) Lt[at + u] = x.v[u];
+    if (Lhi) {
+      Lhi[at + u] = h.v[u];
+      Llo[at + u] = l.v[u];
+    }
+    if (bp.hi) {
+      bp.hi[at + u] = b0.v[u];
+      bp.mid[at + u] = b1.v[u];
+      bp.lo[at + u] = b2.v[u];
+    }
   }
 }
 
@@ -88,13 +133,13 @@ int32_t split_parts(const float* X, int64_t ld, int64_t rows, int cols, float* h
 }
 
 template <typename T>
-int32_t build_ly(const T* Y, int64_t ldy, int64_t m, int k, const int32_t* perm, T* Lt, T* Lp,
+int32_t build_ly(const T* Y, int64_t ldy, int64_t m, int k, const int32_t* pos, T* Lt, T* Lp,
                  int64_t ldl, cudaStream_t s, T* Lhi, T* Llo, Bf16Parts bp) {
-  const int threads = 256;
-  int64_t bx = ceil_div(m, threads);
-  if (bx > 4096) bx = 4096;
-  k_build_ly<T><<<dim3((unsigned)bx, (unsigned)k), threads, 0, s>>>(Y, ldy, m, k, perm, Lt, Lp,
-                                                                   ldl, Lhi, Llo, bp);
+  auto ok = [](const void* p) { return ((uintptr_t)p & 31u) == 0; };  // null counts as aligned
+  const bool vec = ldy % 4 == 0 && ldl % 4 == 0 && ok(Y) && ok(Lt) && ok(Lhi) && ok(Llo) &&
+                   ok(bp.hi) && ok(bp.mid) && ok(bp.lo);
+  k_build_ly<T><<<dim3((unsigned)ceil_div(m, 1024), (unsigned)k), 256, 0, s>>>(
+      Y, ldy, m, pos, Lt, Lp, ldl, Lhi, Llo, bp, vec);
   return last_launch_status();
 }
 template int32_t build_ly<float>(const float*, int64_t, int64_t, int, const int32_t*, float*,
@@ -256,34 +301,43 @@ __global__ void __launch_bounds__(CH_NT, 1) k_chol_cluster(double* __restrict__ 
   cl.sync();
 }
 
-// Inverses of the TB x TB diagonal blocks of the unit lower L (FP64, column-major k x k),
-// one warp per block, column by column (right-looking, no divides); results and L itself
-// converted to the path's type for the triangular solves.
+// Inverses of the TB x TB diagonal blocks of the unit lower L (FP64, column-major k x k), one
+// CTA per block: its first warp computes the inverse, lane j column j (x_i = [i == j] -
+// sum_{t < i} L[i][t] x_t; the FP64 unit takes 64 cycles per warp instruction, so that a column
+// at a time across the lanes cost 20 times the multiply-adds: 33 us at k = 20), the others
+// convert L to the path's type for the triangular solves.
 static constexpr int TB = 32;
 
 template <typename T>
-__global__ void __launch_bounds__(32) k_diag_inv(const double* __restrict__ Lc, int k,
-                                                 LdlOut<T> o) {
-  const int lane = threadIdx.x, b = blockIdx.x;
+__global__ void __launch_bounds__(128) k_diag_inv(const double* __restrict__ Lc, int k,
+                                                  LdlOut<T> o) {
+  __shared__ double Ls[TB][TB + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.x;
   const int b0 = b * TB, bw = min(TB, k - b0);
+  for (int e = threadIdx.x; e < bw * bw; e += 128) {
+    const int i = e % bw, c = e / bw;
+    Ls[i][c] = Lc[(int64_t)(b0 + c) * k + b0 + i];
+  }
+  __syncthreads();
   // this block's columns of L in the path's type, zero-padded to kp x kp, both layouts
-  for (int c = b0; c < b0 + TB; ++c)
+  for (int c = b0 + warp - 1; c >= b0 && c < b0 + TB; c += 3)  // warps 1 to 3
     for (int i = lane; i < o.kp; i += 32) {
       const T v = (c < k && i < k) ? (T)Lc[(int64_t)c * k + i] : (i == c ? T(1) : T(0));
       o.LT[(int64_t)c * o.kp + i] = v;
       o.LR[(int64_t)i * o.kp + c] = v;
     }
-  // column j of the block inverse: x_j = 1, x_i = -sum_{t<i} L[i][t] x_t (lane i owns x_i)
-  for (int j = 0; j < TB; ++j) {
-    double x = (lane == j) ? 1.0 : 0.0;
-    for (int t = j; t < bw; ++t) {
-      const double xt = __shfl_sync(0xffffffffu, x, t);
-      if (lane > t && lane < bw) x = fma(-Lc[(int64_t)(b0 + t) * k + b0 + lane], xt, x);
+  if (warp != 0) return;
+  double x[TB];
+#pragma unroll
+  for (int i = 0; i < TB; ++i) {
+    x[i] = i == lane ? 1.0 : 0.0;
+    if (i < bw) {
+#pragma unroll
+      for (int t = 0; t < i; ++t) x[i] = fma(-Ls[i][t], x[t], x[i]);
     }
-    // W block b row-major (element (lane, j)) and its transpose
-    const T w = (lane < bw && j < bw) ? (T)x : (lane == j ? T(1) : T(0));
-    o.W[(size_t)b * TB * TB + lane * TB + j] = w;
-    o.WT[(size_t)b * TB * TB + j * TB + lane] = w;
+    const T w = (i < bw && lane < bw) ? (T)x[i] : (i == lane ? T(1) : T(0));
+    o.W[(size_t)b * TB * TB + i * TB + lane] = w;
+    o.WT[(size_t)b * TB * TB + lane * TB + i] = w;
   }
 }
 
@@ -745,7 +799,7 @@ int32_t ldl_factor(double* M, int k, const LdlOut<T>& o, int32_t* status, cudaSt
   if (sizeof(T) == sizeof(float) && k <= LC_MAXB * LB)
     return ldl32_cluster(M, k, reinterpret_cast<const LdlOut<float>&>(o), status, s);
   RLU_TRY(ldl_cluster_f64(M, k, o.dinv, status, s));
-  k_diag_inv<T><<<(unsigned)ceil_div(k, TB), 32, 0, s>>>(M, k, o);
+  k_diag_inv<T><<<(unsigned)ceil_div(k, TB), 128, 0, s>>>(M, k, o);
   return last_launch_status();
 }
 bool ldl_factor_supported(int k, bool f32) {
@@ -1049,8 +1103,12 @@ __global__ void __launch_bounds__(RL_NT) k_trsm_rl(LdlOut<T> o, const T* __restr
     // diagonal pass: X_J = W X_J (W = W_J forward, W_J^T backward), 4 x CPT per thread
     T* XJ = Xs + (size_t)J * TB * TC;
     T d[4][CPT] = {};
+    // rows and columns past k are zero and stay so: FP64, whose multiply-adds count, skips
+    // them (in FP32 the variable trip counts cost more: 471 -> 549 us at k = 512)
+    constexpr bool kSkip = sizeof(T) == 8;
+    const int tb = kSkip ? min(TB, k - J * TB) : TB;
 #pragma unroll 8
-    for (int t = 0; t < TB; ++t) {
+    for (int t = 0; t < (kSkip ? (dr < tb ? tb : 0) : TB); ++t) {
       T xv[CPT];
 #pragma unroll
       for (int b = 0; b < CPT; ++b) xv[b] = XJ[t * TC + dc + b];
@@ -1065,7 +1123,8 @@ __global__ void __launch_bounds__(RL_NT) k_trsm_rl(LdlOut<T> o, const T* __restr
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int b = 0; b < CPT; ++b) XJ[(dr + a) * TC + dc + b] = d[a][b];
+      for (int b = 0; b < CPT; ++b)
+        if (!kSkip || dr < tb) XJ[(dr + a) * TC + dc + b] = d[a][b];
     __syncthreads();
     // update pass: rows i0 .. i1 - 1 of X minus (staged rows t of L^T / L) x X_J
     const int i0 = fwd ? (J + 1) * TB : 0, i1 = fwd ? kp : J * TB;
@@ -1074,7 +1133,7 @@ __global__ void __launch_bounds__(RL_NT) k_trsm_rl(LdlOut<T> o, const T* __restr
       const int r0 = st * RG * TR + ug * TR;  // row offset within the updated range
       T acc[TR][4] = {};
 #pragma unroll 4
-      for (int t = 0; t < TB; ++t) {
+      for (int t = 0; t < (kSkip ? tb : TB); ++t) {
         const Vec4<T> x = lds4(XJ + t * TC + uc);
 #pragma unroll
         for (int h = 0; h < TR / 4; ++h) {
@@ -1159,45 +1218,57 @@ template int32_t trsm_ldl<float>(const LdlOut<float>&, const float*, int64_t, in
 template int32_t trsm_ldl<double>(const LdlOut<double>&, const double*, int64_t, int64_t, double*,
                                   int64_t, cudaStream_t, bool);
 
-// L_b (k x k, column-major, ld k): L_b[i][j] = X^T-stored B[i][Q[j]] for i > j, 1 on the
-// diagonal, 0 above. B is row-major k x n (ld ldb).
+// U (k x n, row-major, ld ldu): U[i][j] = B[i][Q[j]] for j >= i, 0 below the diagonal, four
+// rows a thread (they share Q[j], and their gathers are in flight together). Grid rows past
+// U's write L_b (k x k): L_b[i][j] = B[i][Q[j]] for i > j, 1 on the diagonal, 0 above, as it is
+// (Lb, column-major, ld k) and / or as its TF32 parts (Lbh, Lbl, ld ldh). B is row-major k x n.
 template <typename T>
-__global__ void k_gather_lb(const T* __restrict__ B, int64_t ldb, const int32_t* __restrict__ Q,
-                            int k, T* __restrict__ Lb) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)k * k;
-       e += (int64_t)gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(256) k_gather_lb_u(const T* __restrict__ B, int64_t ldb,
+                                                     const int32_t* __restrict__ Q, int k,
+                                                     int64_t n, T* __restrict__ Lb,
+                                                     T* __restrict__ Lbh, T* __restrict__ Lbl,
+                                                     int64_t ldh, T* __restrict__ U, int64_t ldu) {
+  const int ub = (k + 3) / 4;  // grid rows of U
+  const int64_t x = blockIdx.x * 256ll + threadIdx.x;
+  if ((int)blockIdx.y < ub) {
+    const int i0 = 4 * (int)blockIdx.y;
+    for (int64_t j = x; j < n; j += gridDim.x * 256ll) {
+      const int64_t q = Q[j];
+      T v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        v[u] = i0 + u < k && j >= i0 + u ? B[(int64_t)(i0 + u) * ldb + q] : T(0);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i0 + u < k) U[(int64_t)(i0 + u) * ldu + j] = v[u];
+    }
+    return;
+  }
+  const int64_t threads = (int64_t)(gridDim.y - ub) * gridDim.x * 256;
+  for (int64_t e = ((int64_t)(blockIdx.y - ub) * gridDim.x) * 256 + x; e < (int64_t)k * k;
+       e += threads) {
     const int j = (int)(e / k), i = (int)(e % k);
-    Lb[e] = i > j ? B[(int64_t)i * ldb + Q[j]] : (i == j ? T(1) : T(0));
+    const T v = i > j ? B[(int64_t)i * ldb + Q[j]] : (i == j ? T(1) : T(0));
+    if (Lb) Lb[e] = v;
+    if (Lbh) tf32_split(v, Lbh, Lbl, (int64_t)j * ldh + i);
   }
 }
 
-// U (k x n, row-major, ld ldu): U[i][j] = B[i][Q[j]] for j >= i, 0 below the diagonal.
 template <typename T>
-__global__ void k_gather_u(const T* __restrict__ B, int64_t ldb, const int32_t* __restrict__ Q,
-                           int k, int64_t n, T* __restrict__ U, int64_t ldu) {
-  const int i = blockIdx.y;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
-       j += (int64_t)gridDim.x * blockDim.x)
-    U[(int64_t)i * ldu + j] = j >= i ? B[(int64_t)i * ldb + Q[j]] : T(0);
-}
-
-template <typename T>
-int32_t gather_lb_u(const T* B, int64_t ldb, const int32_t* Q, int k, int64_t n, T* Lb, T* U,
-                    int64_t ldu, cudaStream_t s) {
-  const int threads = 256;
-  int64_t blocks = ceil_div((int64_t)k * k, threads);
-  if (blocks > 1024) blocks = 1024;
-  k_gather_lb<T><<<(unsigned)blocks, threads, 0, s>>>(B, ldb, Q, k, Lb);
-  RLU_TRY(last_launch_status());
-  int64_t bx = ceil_div(n, threads);
+int32_t gather_lb_u(const T* B, int64_t ldb, const int32_t* Q, int k, int64_t n, T* Lb, T* Lbh,
+                    T* Lbl, int64_t ldh, T* U, int64_t ldu, cudaStream_t s) {
+  int64_t bx = ceil_div(n, 256);
   if (bx > 1024) bx = 1024;
-  k_gather_u<T><<<dim3((unsigned)bx, (unsigned)k), threads, 0, s>>>(B, ldb, Q, k, n, U, ldu);
+  const unsigned lrows = (unsigned)std::min<int64_t>(ceil_div((int64_t)k * k, 256 * bx), 64);
+  k_gather_lb_u<T><<<dim3((unsigned)bx, (unsigned)ceil_div(k, 4) + lrows), 256, 0, s>>>(
+      B, ldb, Q, k, n, Lb, Lbh, Lbl, ldh, U, ldu);
   return last_launch_status();
 }
 template int32_t gather_lb_u<float>(const float*, int64_t, const int32_t*, int, int64_t, float*,
-                                    float*, int64_t, cudaStream_t);
+                                    float*, float*, int64_t, float*, int64_t, cudaStream_t);
 template int32_t gather_lb_u<double>(const double*, int64_t, const int32_t*, int, int64_t,
-                                     double*, double*, int64_t, cudaStream_t);
+                                     double*, double*, double*, int64_t, double*, int64_t,
+                                     cudaStream_t);
 
 // Contiguous copy with stride change: dst (rows x cols, column-major ld ldd) <- src (ld lds).
 template <typename T>

@@ -18,8 +18,10 @@ struct Bf16Parts {
 int32_t split_parts(const float* X, int64_t ld, int64_t rows, int cols, float* hi, float* lo,
                     Bf16Parts bp, cudaStream_t s, int64_t ldo = 0);
 
+// From the factored Y (swap-free) and its rows' positions: Lp = L_y's first k columns in pivot
+// order, Lt = L~ = P^T L_y and its splits (null outputs are skipped).
 template <typename T>
-int32_t build_ly(const T* Y, int64_t ldy, int64_t m, int k, const int32_t* perm, T* Lt, T* Lp,
+int32_t build_ly(const T* Y, int64_t ldy, int64_t m, int k, const int32_t* pos, T* Lt, T* Lp,
                  int64_t ldl, cudaStream_t s, T* Lhi = nullptr, T* Llo = nullptr,
                  Bf16Parts bp = Bf16Parts{});
 
@@ -51,9 +53,11 @@ template <typename T>
 int32_t trsm_ldl(const LdlOut<T>& o, const T* C, int64_t ldc, int64_t n, T* B, int64_t ldb,
                  cudaStream_t s, bool narrow = false);
 
+// L_b (k x k, column-major, ld k) and / or its exact TF32 parts (ld ldh; null: skipped), and
+// U, from the factored B.
 template <typename T>
-int32_t gather_lb_u(const T* B, int64_t ldb, const int32_t* Q, int k, int64_t n, T* Lb, T* U,
-                    int64_t ldu, cudaStream_t s);
+int32_t gather_lb_u(const T* B, int64_t ldb, const int32_t* Q, int k, int64_t n, T* Lb, T* Lbh,
+                    T* Lbl, int64_t ldh, T* U, int64_t ldu, cudaStream_t s);
 
 template <typename T>
 int32_t copy_cm(const T* src, int64_t lds, T* dst, int64_t ldd, int64_t rows, int64_t cols,
