@@ -24,6 +24,7 @@
 #include "common.cuh"
 #include "gemm_simt.cuh"
 #include "panel_lu.cuh"
+#include "side.cuh"
 #include "small.cuh"
 #include "umma.cuh"
 #include "../../include/rlu_fast.h"
@@ -1043,46 +1044,52 @@ static int32_t fast_factor(const FastPlan& p, const float* A, int64_t m, int64_t
   o.dinv = reinterpret_cast<double*>(ws + p.off_dinv);
   o.k = k2;
   o.kp = p.kp;
-  RLU_TRY(ldl_factor<float>(Mre, k2, o, status, s));
-  {
-    const int64_t ldv = 2 * (int64_t)l;
-    int32_t st;
-    switch (p.ns) {
-      case 1: st = wsolve_launch<1>(V, ldv, k, l, Y, l, Wst, l, s); break;
-      case 2: st = wsolve_launch<2>(V, ldv, k, l, Y, l, Wst, l, s); break;
-      case 4: st = wsolve_launch<4>(V, ldv, k, l, Y, l, Wst, l, s); break;
-      case 8: st = wsolve_launch<8>(V, ldv, k, l, Y, l, Wst, l, s); break;
-      default: st = wsolve_launch<16>(V, ldv, k, l, Y, l, Wst, l, s); break;
+  // the LDL^T (a cluster of 8 CTAs) runs beside W and C (measured at 4096^2, k = 256: 220 us
+  // beside about 125)
+  auto form_c = [&]() -> int32_t {
+    {
+      const int64_t ldv = 2 * (int64_t)l;
+      int32_t st;
+      switch (p.ns) {
+        case 1: st = wsolve_launch<1>(V, ldv, k, l, Y, l, Wst, l, s); break;
+        case 2: st = wsolve_launch<2>(V, ldv, k, l, Y, l, Wst, l, s); break;
+        case 4: st = wsolve_launch<4>(V, ldv, k, l, Y, l, Wst, l, s); break;
+        case 8: st = wsolve_launch<8>(V, ldv, k, l, Y, l, Wst, l, s); break;
+        default: st = wsolve_launch<16>(V, ldv, k, l, Y, l, Wst, l, s); break;
+      }
+      RLU_TRY(st);
     }
-    RLU_TRY(st);
-  }
-  k_frlu_gather_aj<<<dim3((unsigned)std::min<int64_t>(ceil_div(n, 256), 64), (unsigned)l), 256, 0, s>>>(
-      A, lda, (int)n, P, AJ, p.ldn);
-  RLU_TRY(last_launch_status());
-  if (p.tc) {  // C^T = A(J,:)^T W^T: A(J,:) as the raw n-contiguous operand, W's TF32 parts
-    float* Wh = reinterpret_cast<float*>(ws + p.off_Wh);
-    float* Wl = reinterpret_cast<float*>(ws + p.off_Wl);
-    RLU_TRY(split_parts(Wst, l, l, k2, Wh, Wl, Bf16Parts{}, s));
-    Umma3Op op{};
-    op.A0 = AJ;
-    op.lda = p.ldn;
-    op.B0 = Wh;
-    op.B1 = Wl;
-    op.ldb = l;
-    op.M = n;
-    op.N = k2;
-    op.K = l;
-    op.out = Cst;
-    op.ldo = p.ldn;
-    op.out_colmajor = true;
-    op.splits = umma3_splits(n, l, k2);
-    op.partial = reinterpret_cast<float*>(ws + p.off_part2);
-    op.status = status;
-    RLU_TRY(umma3_gemm(U3_MODE_C3, op, s));
-  } else {
-    GemmOp op{Wst, l, true, AJ, p.ldn, false, Cst, p.ldn, true, k2, n, l, 1, nullptr, false};
-    RLU_TRY((gemm_simt<float, float>(op, s)));
-  }
+    k_frlu_gather_aj<<<dim3((unsigned)std::min<int64_t>(ceil_div(n, 256), 64), (unsigned)l), 256, 0, s>>>(
+        A, lda, (int)n, P, AJ, p.ldn);
+    RLU_TRY(last_launch_status());
+    if (p.tc) {  // C^T = A(J,:)^T W^T: A(J,:) as the raw n-contiguous operand, W's TF32 parts
+      float* Wh = reinterpret_cast<float*>(ws + p.off_Wh);
+      float* Wl = reinterpret_cast<float*>(ws + p.off_Wl);
+      RLU_TRY(split_parts(Wst, l, l, k2, Wh, Wl, Bf16Parts{}, s));
+      Umma3Op op{};
+      op.A0 = AJ;
+      op.lda = p.ldn;
+      op.B0 = Wh;
+      op.B1 = Wl;
+      op.ldb = l;
+      op.M = n;
+      op.N = k2;
+      op.K = l;
+      op.out = Cst;
+      op.ldo = p.ldn;
+      op.out_colmajor = true;
+      op.splits = umma3_splits(n, l, k2);
+      op.partial = reinterpret_cast<float*>(ws + p.off_part2);
+      op.status = status;
+      RLU_TRY(umma3_gemm(U3_MODE_C3, op, s));
+    } else {
+      GemmOp op{Wst, l, true, AJ, p.ldn, false, Cst, p.ldn, true, k2, n, l, 1, nullptr, false};
+      RLU_TRY((gemm_simt<float, float>(op, s)));
+    }
+    return RLU_OK;
+  };
+  RLU_TRY(run_beside(s, [&](cudaStream_t hs) { return ldl_factor<float>(Mre, k2, o, status, hs); },
+                     form_c));
   RLU_TRY(trsm_ldl<float>(o, Cst, p.ldn, n, Bst, p.ldn, s, ceil_div(n, 64) < sm_count()));
   // step 7: B Q = L_b U_b through the Crout LU of B^T
   k_frlu_pack_bt<<<dim3((unsigned)ceil_div(n, 32), (unsigned)ceil_div(k, 32)), dim3(32, 8), 0, s>>>(

@@ -12,6 +12,7 @@
 // LDL^T and the products.
 #include "common.cuh"
 #include "gemm_simt.cuh"
+#include "side.cuh"
 #include "small.cuh"
 
 namespace rlu {
@@ -144,23 +145,25 @@ static int32_t lstsq_t(const LsPlan& p, int64_t m, int64_t n, int k, const int32
   o.k = k;
   o.kp = p.kp;
   if (info) RLU_TRY(info_init(info, s));
-  // c = P b
-  int64_t bx = ceil_div(m, 256);
-  if (bx > 1024) bx = 1024;
-  k_gather_rows<T><<<dim3((unsigned)bx, (unsigned)nrhs), 256, 0, s>>>(b, ldb, P, m, c, p.ldc);
-  RLU_TRY(last_launch_status());
-  // M = L^T L (FP64), its LDL^T
+  // M = L^T L (FP64)
   {
     GemmOp op{L, ldl, true, L, ldl, true, M, k, true, k, k, m, p.split, part, false};
     RLU_TRY((gemm_simt<T, double>(op, s)));
   }
-  RLU_TRY(ldl_factor<T>(M, k, o, info ? &info->status : nullptr, s));
-  // Cr = L^T c (k x nrhs, row-major), y = M^{-1} Cr
-  {
+  // its LDL^T (one CTA, or a cluster) beside c = P b and Cr = L^T c (k x nrhs, row-major)
+  auto form_c = [&]() -> int32_t {
+    int64_t bx = ceil_div(m, 256);
+    if (bx > 1024) bx = 1024;
+    k_gather_rows<T><<<dim3((unsigned)bx, (unsigned)nrhs), 256, 0, s>>>(b, ldb, P, m, c, p.ldc);
+    RLU_TRY(last_launch_status());
     GemmOp op{L, ldl, true, c, p.ldc, true, Cr, p.nr, true, k, nrhs, m, p.split, part, false};
-    RLU_TRY((gemm_simt<T, T>(op, s)));
-  }
-  RLU_TRY(trsm_ldl<T>(o, Cr, p.nr, nrhs, Yk, p.nr, s));
+    return gemm_simt<T, T>(op, s);
+  };
+  RLU_TRY(run_beside(
+      s, [&](cudaStream_t hs) { return ldl_factor<T>(M, k, o, info ? &info->status : nullptr, hs); },
+      form_c));
+  // y = M^{-1} Cr; up to 32 right-hand sides leave half of a 64-column CTA idle
+  RLU_TRY(trsm_ldl<T>(o, Cr, p.nr, nrhs, Yk, p.nr, s, nrhs <= 32));
   // z_1 = U_1^{-1} y, x = Q (z_1, 0)
   k_upper_solve<T><<<(unsigned)nrhs, US_T, sizeof(T) * (size_t)k, s>>>(
       U, ldu, k, n, Q, Yk, p.nr, x, ldx, info ? &info->first_zero_pivot_b : nullptr);

@@ -19,6 +19,7 @@
 #include "gemm_simt.cuh"
 #include "panel_lu.cuh"
 #include "residual.cuh"
+#include "side.cuh"
 #include "small.cuh"
 #include "umma.cuh"
 
@@ -55,15 +56,7 @@ int sm_count() {
   return n;
 }
 
-// Helper stream and fork/join events of one caller stream on one device (created on first
-// use), so that concurrent factorizations on different streams keep separate helpers.
-struct SideStream {
-  cudaStream_t side = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
-  std::mutex mu;
-};
-
-static int32_t side_stream(cudaStream_t main, SideStream** out) {
+int32_t side_stream(cudaStream_t main, SideStream** out) {
   static std::mutex table_mu;
   static std::map<std::pair<int, cudaStream_t>, SideStream*> table;
   int dev = 0;
@@ -558,16 +551,12 @@ static int32_t factor_t(const Plan& p, const void* Av, int64_t lda, uint64_t see
     RLU_TRY((gemm_simt<T, double>(op, s)));
   }
   RLU_TRY(tm.rec(4, true, s));
-  SideStream* ss = nullptr;
-  RLU_TRY(side_stream(s, &ss));
-  {
-    std::lock_guard<std::mutex> lock(ss->mu);
-    RLU_CUDA_TRY(cudaEventRecord(ss->fork, s));
-    RLU_CUDA_TRY(cudaStreamWaitEvent(ss->side, ss->fork, 0));
-    RLU_TRY(tm.rec(5, false, ss->side));
-    RLU_TRY(ldl_factor<T>(M, k, ldl, info ? &info->status : nullptr, ss->side));
-    RLU_TRY(tm.rec(5, true, ss->side));
-    RLU_CUDA_TRY(cudaEventRecord(ss->join, ss->side));
+  auto factor_gram = [&](cudaStream_t hs) -> int32_t {
+    RLU_TRY(tm.rec(5, false, hs));
+    RLU_TRY(ldl_factor<T>(M, k, ldl, info ? &info->status : nullptr, hs));
+    return tm.rec(5, true, hs);
+  };
+  auto product_c = [&]() -> int32_t {
     // C = L~^T A (k x n, row-major)
     RLU_TRY(tm.rec(6, false, s));
     if (bf16) {  // C = L~^T A with L~ in three BF16 parts and BF16 A
@@ -609,9 +598,9 @@ static int32_t factor_t(const Plan& p, const void* Av, int64_t lda, uint64_t see
       GemmOp op{Lt, p.ldl, true, A, lda, false, Cb, p.ldb, true, k, n, m, p.split_c, part, false};
       RLU_TRY((gemm_simt<T, T>(op, s)));
     }
-    RLU_TRY(tm.rec(6, true, s));
-    RLU_CUDA_TRY(cudaStreamWaitEvent(s, ss->join, 0));
-  }
+    return tm.rec(6, true, s);
+  };
+  RLU_TRY(run_beside(s, factor_gram, product_c));
   // B = M^{-1} C = L^{-T} D^{-1} L^{-1} C
   RLU_TRY(tm.rec(7, false, s));
   // FP64: 32 columns a CTA where 64 would leave SMs' FP64 units idle (and the narrow form fits)
