@@ -470,6 +470,9 @@ __device__ __forceinline__ void lu_reg_body(const LuArgs& a) {
     // records are in flight, and what is rare (ties, zeros, Inf and NaN, the two rows whose
     // positions change) sits behind branches that are seldom taken.
     using K = key_t<T>;
+    // FP64 multiply-adds (64 cycles each) are worth a branch around dead columns, where the
+    // branches cost no spills
+    constexpr bool kSlow = std::is_same<T, double>::value && RT <= 2;
     const uint32_t recv_a = smem_u32(&sh.recv[0][0][0]);
     const uint32_t ub_a = smem_u32(ub);
     T x[RT][LB];        // rows r0 + tid + s NC: the block's columns from the current one on
@@ -715,7 +718,8 @@ __device__ __forceinline__ void lu_reg_body(const LuArgs& a) {
         pnz = nz;
         if (CROUT) {
 #pragma unroll
-          for (int c = 1; c < LB; ++c) P[c] = P[c] * prp;
+          for (int c = 1; c < LB; ++c)
+            if (!kSlow || c < LB - i) P[c] = P[c] * prp;
         }
         // positions after the exchange of positions j and the winner's
         const int wpos = wpr >> 16;
@@ -756,7 +760,8 @@ __device__ __forceinline__ void lu_reg_body(const LuArgs& a) {
         for (int s = 0; s < RT; ++s) {
           x[s][0] = m[s] != T(0) ? fma(-m[s], P[1], x[s][1]) : x[s][1];
 #pragma unroll
-          for (int c = 1; c + 1 < LB; ++c) x[s][c] = fma(-m[s], P[c + 1], x[s][c + 1]);
+          for (int c = 1; c + 1 < LB; ++c)
+            if (!kSlow || c + 1 < LB - i) x[s][c] = fma(-m[s], P[c + 1], x[s][c + 1]);
         }
       }
       store_step(b0 + bw - 1, Xj - ldx, rem > 0 || tail);
@@ -826,7 +831,8 @@ __device__ __forceinline__ void lu_reg_body(const LuArgs& a) {
           for (int s = 0; s < RT; ++s) {
             const T mq = xb[q * rs + tid + s * NC];
 #pragma unroll
-            for (int c = 0; c < LB; ++c) x[s][c] = fma(-mq, uv[c], x[s][c]);
+            for (int c = 0; c < LB; ++c)
+              if (!kSlow || c < rem) x[s][c] = fma(-mq, uv[c], x[s][c]);
           }
         }
         __syncwarp();  // uc is free for the next block
@@ -1250,8 +1256,8 @@ static int32_t launch_reg_t(const LuArgs& a, cudaStream_t s, bool* launched) {
   } else {
     RLU_LU_TRY(16 * 32, 1, 32, 36);
     RLU_LU_TRY(16 * 64, 1, 64, 36);
-    RLU_LU_TRY(16 * 128, 1, 128, 36);
-    RLU_LU_TRY(16 * 256, 2, 128, 36);
+    RLU_LU_TRY(16 * 128, 1, 128, 76);
+    RLU_LU_TRY(16 * 256, 2, 128, 76);
     RLU_LU_TRY(16 * 512, 4, 128, 36);
     RLU_LU_TRY(16 * 1024, 4, 256, 18);
     RLU_LU_TRY(16 * 2048, 8, 256, 8);
