@@ -178,7 +178,6 @@ struct rlu_batch {
   int launches = 0;
   // tensor-core rings of the mixed precision (Y = A G, C = L~^T A)
   int u3y_stages = 0, u3y_stage_bytes = 0, u3c_stages = 0, u3c_stage_bytes = 0;
-  int ts_first[4] = {}, ts_count[4] = {};  // small-k substitution tiles per bucket of k
   rlu_batch_options opt{};
   rlu::LuFork lu_fork{};  // helper streams: the LU groups run side by side
   bool have_fork = false;
@@ -319,7 +318,7 @@ extern "C" int32_t rlu_batch_create(const rlu_problem* problems, int32_t count, 
     lub_all[(size_t)i] = u;
     float* Lhi = mixed ? reinterpret_cast<float*>(ws + L.Lhi) : nullptr;
     float* Llo = mixed ? reinterpret_cast<float*>(ws + L.Llo) : nullptr;
-    build[(size_t)i] = BuildJob{Y, L.ldy, p.m, p.k, p.P, Lt, Lp, L.ldl, Lhi, Llo};
+    build[(size_t)i] = BuildJob{Y, L.ldy, p.m, p.k, p.P, pos, Lt, Lp, L.ldl, Lhi, Llo};
     if (mixed) {  // tensor-core records of Y = A G and C^T = A^T L~
       Umma3Op op{};
       op.A0 = static_cast<const float*>(p.A);
@@ -366,6 +365,9 @@ extern "C" int32_t rlu_batch_create(const rlu_problem* problems, int32_t count, 
     b->max_l = std::max(b->max_l, p.l);
     b->max_kp = std::max(b->max_kp, L.kp);
   }
+  // the Gram matrices' sums run over m in order: the longest first
+  std::stable_sort(gg.begin(), gg.end(),
+                   [](const GemmArgs& x, const GemmArgs& y) { return x.K > y.K; });
   // LU records grouped by cluster size
   auto group = [&](const std::vector<LuArgs>& all, const std::vector<int>& gof, int* first,
                    int* cnt, std::vector<LuArgs>& sorted) {
@@ -407,15 +409,12 @@ extern "C" int32_t rlu_batch_create(const rlu_problem* problems, int32_t count, 
     tt.reserve((size_t)t.n_tiles_t);
     tl.reserve((size_t)t.n_tiles_l);
     const int cw = t.small_k ? 128 : 64;
-    // small k: the substitution's tiles grouped by the bucket of k (one launch each)
-    for (int bkt = 0; bkt < (t.small_k ? 4 : 1); ++bkt) {
-      if (t.small_k) b->ts_first[bkt] = (int)tt.size();
+    // small k: the substitution's tiles by the bucket of k, the longest chains first
+    for (int bkt = t.small_k ? 3 : 0; bkt >= 0; --bkt)
       for (int i = 0; i < count; ++i) {
         if (t.small_k && trsm_small_bucket(problems[i].k) != bkt) continue;
         for (int cb = 0; cb < (int)ceil_div(problems[i].n, cw); ++cb) tt.push_back(make_int2(i, cb));
       }
-      if (t.small_k) b->ts_count[bkt] = (int)tt.size() - b->ts_first[bkt];
-    }
     for (int i = 0; i < count && t.small_k; ++i)
       for (int rb = 0; rb < (int)ceil_div(problems[i].m, 256); ++rb) tl.push_back(make_int2(i, rb));
     if (st == RLU_OK) st = up(t.trsm_tiles, tt.data(), tt.size() * sizeof(int2));
@@ -456,9 +455,7 @@ extern "C" int32_t rlu_batch_create(const rlu_problem* problems, int32_t count, 
   }
   int groups = 0;
   for (int g = 1; g < kLuGroups; ++g) groups += (b->count_y[g] > 0) + (b->count_b[g] > 0);
-  int buckets = 0;  // the small-k substitution: one launch per nonempty bucket of k
-  for (int bkt = 0; bkt < 4; ++bkt) buckets += b->ts_count[bkt] > 0;
-  b->launches = 10 + groups + (t.small_k && buckets > 1 ? buckets - 1 : 0);
+  b->launches = 10 + groups;
   *out = b;
   return RLU_OK;
 }
@@ -507,8 +504,7 @@ extern "C" int32_t rlu_factor_batched(rlu_batch* b, void* stream) {
                                              b->opt.gemm_tile_c)));
   if (t.small_k)
     RLU_TRY(trsm_small_batched(reinterpret_cast<const TrsmJob*>(ws + t.trsm),
-                               reinterpret_cast<const int2*>(ws + t.trsm_tiles), b->ts_first,
-                               b->ts_count, s));
+                               reinterpret_cast<const int2*>(ws + t.trsm_tiles), t.n_tiles_t, s));
   else
     RLU_TRY(trsm_batched(reinterpret_cast<const TrsmJob*>(ws + t.trsm),
                          reinterpret_cast<const int2*>(ws + t.trsm_tiles), t.n_tiles_t, b->max_kp,

@@ -20,7 +20,8 @@ struct BuildJob {  // step 4: L_y (pivot order, Lp) and L~ = P^T L_y (Lt), both 
   const float* Y;
   int64_t ldy, m;
   int k;
-  const int32_t* perm;
+  const int32_t* perm;  // row of Y at each position
+  const int32_t* pos;   // and the position of each row
   float* Lt;
   float* Lp;
   int64_t ldl;
@@ -63,13 +64,12 @@ int32_t trsm_batched(const TrsmJob* jobs_dev, const int2* tiles_dev, int ntiles,
                      cudaStream_t s);
 int32_t gather_batched(const GatherJob* jobs_dev, int count, int max_k, int64_t max_n,
                        cudaStream_t s);
-// k <= 64: the substitution one thread per column over (problem, 128-column block) tiles,
-// grouped by the bucket of k (trsm_small_bucket: 0..3 for k <= 16, 32, 48, 64; tiles of
-// bucket b at first[b] .. first[b] + count[b] - 1, one launch per nonempty bucket), and
-// L = L_y L_b one thread per row over (problem, 256-row block) tiles
+// k <= 64: the substitution one thread per column over (problem, 128-column block) tiles, in any
+// order (the larger buckets of k first is best: trsm_small_bucket is 0..3 for k <= 16, 32, 48,
+// 64), and L = L_y L_b two rows per thread over (problem, 256-row block) tiles
 int trsm_small_bucket(int k);
-int32_t trsm_small_batched(const TrsmJob* jobs_dev, const int2* tiles_dev, const int* first,
-                           const int* count, cudaStream_t s);
+int32_t trsm_small_batched(const TrsmJob* jobs_dev, const int2* tiles_dev, int ntiles,
+                           cudaStream_t s);
 int32_t lmul_batched(const GemmArgs* jobs_dev, const int2* tiles_dev, int ntiles, cudaStream_t s);
 // k <= 64: the Gram M = L~^T L~ (FP64 out, FP32 accumulation), one CTA per problem
 int32_t gram_small_batched(const GemmArgs* jobs_dev, int count, cudaStream_t s);

@@ -846,6 +846,12 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
+// the first `bytes` of the 16 from src, zeros after them
+__device__ __forceinline__ void cp_async16_part(void* dst, const void* src, int bytes) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(bytes)
+               : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() {
   asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
@@ -1312,34 +1318,49 @@ int32_t info_init(rlu_info* info, cudaStream_t s) {
 }
 
 // ---- batched launchers --------------------------------------------------------------------
-// CTA (problem blockIdx.x, column group blockIdx.y): columns c = y, y + gridDim.y, ... of
-// L_y / L~ (m rows each) in a loop, so that the grid holds no CTAs for the rows small
-// problems do not have. The CTA first inverts the permutation in shared memory
-// (pinv[perm[p]] = p), so that it walks the rows of L~ = P^T L_y (and of Y and the TF32
-// split) in order: only the writes of L_y in pivot order are scattered.
-__global__ void k_build_ly_batched(const BuildJob* __restrict__ jobs) {
-  extern __shared__ int bl_pinv[];  // [m]
+// The batch's gathers by row or column index go through shared memory: a warp that reads or
+// writes 32 scattered words of global memory takes 32 sectors, a few shared-memory cycles
+// here. Columns (L_y) or rows (U) are staged BG at a time: four while the longest of the batch
+// keeps that within 32 KB, so that several CTAs still share an SM, else one.
+static constexpr int64_t BG_LONG = 2048;
+
+// CTA (problem blockIdx.x, group blockIdx.y) of L_y and L~: BG columns of Y at a time, read once
+// in row order, which is L~'s order (row r is L_y's row pos[r]), with the TF32 split; the rows
+// of L_y in pivot order come from the staged columns. Bound by its five passes over m x k
+// floats: 58 us for 512 problems of m <= 2048, k <= 64, 75 with the stores of L_y scattered
+// over memory.
+template <int BG>
+__global__ void __launch_bounds__(256) k_build_ly_batched(const BuildJob* __restrict__ jobs) {
+  extern __shared__ float bl_col[];  // [BG][m]
   const BuildJob& j = jobs[blockIdx.x];
-  const int64_t m = j.m;
-  const int k = j.k;
-  // entries outside [0, m) (an LU that stopped early) leave -1 and are skipped
-  for (int64_t r = threadIdx.x; r < m; r += blockDim.x) bl_pinv[r] = -1;
-  __syncthreads();
-  for (int64_t p = threadIdx.x; p < m; p += blockDim.x) {
-    const int q = j.perm[p];
-    if (q >= 0 && q < m) bl_pinv[q] = (int)p;
-  }
-  __syncthreads();
-  for (int c = blockIdx.y; c < k; c += gridDim.y) {
-#pragma unroll 4
-    for (int64_t r = threadIdx.x; r < m; r += blockDim.x) {
-      const int p = bl_pinv[r];
-      if (p < 0) continue;
-      const float v = (c < p) ? j.Y[(int64_t)c * j.ldy + r] : (c == p ? 1.f : 0.f);
-      j.Lt[(int64_t)c * j.ldl + r] = v;
-      if (j.Lhi) tf32_split(v, j.Lhi, j.Llo, (int64_t)c * j.ldl + r);
-      j.Lp[(int64_t)c * j.ldl + p] = v;
+  const int m = (int)j.m, k = j.k;
+  for (int c0 = BG * blockIdx.y; c0 < k; c0 += BG * gridDim.y) {
+    const float* Yc = j.Y + (int64_t)c0 * j.ldy;
+    const int64_t at = (int64_t)c0 * j.ldl;
+    for (int r = threadIdx.x; r < m; r += blockDim.x) {
+      const int p = j.pos[r];
+      float v[BG];
+#pragma unroll
+      for (int u = 0; u < BG; ++u) v[u] = c0 + u < k ? Yc[u * j.ldy + r] : 0.f;
+#pragma unroll
+      for (int u = 0; u < BG; ++u) {
+        bl_col[u * m + r] = v[u];
+        if (c0 + u >= k || p < 0 || p >= m) continue;  // an LU that stopped early
+        const float w = c0 + u < p ? v[u] : (c0 + u == p ? 1.f : 0.f);
+        j.Lt[at + u * j.ldl + r] = w;
+        if (j.Lhi) tf32_split(w, j.Lhi, j.Llo, at + u * j.ldl + r);
+      }
     }
+    __syncthreads();
+    for (int p = threadIdx.x; p < m; p += blockDim.x) {
+      const int r = j.perm[p];
+      if (r < 0 || r >= m) continue;
+#pragma unroll
+      for (int u = 0; u < BG; ++u)
+        if (c0 + u < k)
+          j.Lp[at + u * j.ldl + p] = c0 + u < p ? bl_col[u * m + r] : (c0 + u == p ? 1.f : 0.f);
+    }
+    __syncthreads();
   }
 }
 
@@ -1347,74 +1368,93 @@ int32_t build_ly_batched(const BuildJob* jobs_dev, int count, int64_t max_m, int
                          cudaStream_t s) {
   if (count <= 0) return RLU_OK;
   (void)max_k;
-  const size_t smem = (size_t)max_m * sizeof(int);
-  RLU_CUDA_TRY(cudaFuncSetAttribute(k_build_ly_batched, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const bool four = max_m <= BG_LONG;
+  const auto kernel = four ? k_build_ly_batched<4> : k_build_ly_batched<1>;
+  const size_t smem = (size_t)max_m * sizeof(float) * (four ? 4 : 1);
+  RLU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem));
-  k_build_ly_batched<<<dim3((unsigned)count, 8), 256, smem, s>>>(jobs_dev);
+  kernel<<<dim3((unsigned)count, 8), 256, smem, s>>>(jobs_dev);
   return last_launch_status();
 }
 
 // Gram M = L~^T L~ (k x k, FP64 out, FP32 accumulation) for k <= 64: one CTA per problem;
-// thread t holds the 4 x 4 block (4 (t / 16), 4 (t % 16)) of M; 32-row chunks of L~ are
-// staged row-major in shared memory.
-static constexpr int GS_CHUNK = 32;
+// thread t holds the t-th 4 x 4 block of the lower triangle (M is symmetric to the bit: the
+// same products in the same order) and stores it on both sides. A sum runs over m in order, so
+// the longest problem's chain bounds the kernel: 64 rows of every column are staged at a time,
+// two chunks ahead of the one in use, and a step of four rows is eight 16-byte loads for 64
+// multiply-adds. The 16-byte pieces of a column are stored at their number xor column / 4, so
+// that eight neighbouring blocks read different banks. 99 us for 512 problems of m <= 2048,
+// k <= 64; full squares, 32-row chunks and one chunk ahead took 155.
 static constexpr int GS_KMAX = 64;
-__global__ void __launch_bounds__(256) k_gram_small_batched(const GemmArgs* __restrict__ jobs) {
-  __shared__ __align__(16) float S[GS_CHUNK][GS_KMAX + 4];
+static constexpr int GS_ROWS = 64;
+static constexpr int GS_STAGES = 3;
+static constexpr int GS_NT = 160;  // 136 blocks at k = 64
+__global__ void __launch_bounds__(GS_NT) k_gram_small_batched(const GemmArgs* __restrict__ jobs) {
+  __shared__ __align__(16) float S[GS_STAGES][GS_KMAX][GS_ROWS];
   const GemmArgs& g = jobs[blockIdx.x];
-  const int k = (int)g.N;
-  const int64_t m = g.K;
+  const int k = (int)g.N, m = (int)g.K, nt = (k + 3) / 4, tid = threadIdx.x;
   const float* Lt = static_cast<const float*>(g.A);
-  const int ti = threadIdx.x / 16, tj = threadIdx.x % 16;
-  const bool active = 4 * ti < k && 4 * tj < k;
-  float acc[4][4] = {};
-  constexpr int PER = GS_CHUNK * GS_KMAX / 256;  // staged values per thread and chunk
-  float nxt[PER];                                // the next chunk, loaded ahead
-  auto load_chunk = [&](int64_t r0) {
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      const int e = threadIdx.x + 256 * u;
-      const int c = e / GS_CHUNK, rr = e % GS_CHUNK;  // column c, row r0 + rr (coalesced in rr)
-      nxt[u] = (c < k && r0 + rr < m) ? Lt[(int64_t)c * g.lda + r0 + rr] : 0.f;
-    }
-  };
-  load_chunk(0);
-  for (int64_t r0 = 0; r0 < m; r0 += GS_CHUNK) {
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      const int e = threadIdx.x + 256 * u;
-      S[e % GS_CHUNK][e / GS_CHUNK] = nxt[u];
-    }
-    __syncthreads();
-    if (r0 + GS_CHUNK < m) load_chunk(r0 + GS_CHUNK);
-    if (active) {
-#pragma unroll 8
-      for (int rr = 0; rr < GS_CHUNK; ++rr) {
-        const float4 a = *reinterpret_cast<const float4*>(&S[rr][4 * ti]);
-        const float4 b = *reinterpret_cast<const float4*>(&S[rr][4 * tj]);
-        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-#pragma unroll
-          for (int y = 0; y < 4; ++y) acc[x][y] = fmaf(av[x], bv[y], acc[x][y]);
+  const int64_t lda = g.lda;
+  int ti = 0;
+  while ((ti + 1) * (ti + 2) / 2 <= tid) ++ti;
+  const int tj = tid - ti * (ti + 1) / 2;
+  const int chunks = (m + GS_ROWS - 1) / GS_ROWS;
+  auto stage = [&](int ch) {
+    if (ch < chunks) {
+      float(*D)[GS_ROWS] = S[ch % GS_STAGES];
+      for (int e = tid; e < 4 * nt * (GS_ROWS / 4); e += GS_NT) {
+        const int c = e / (GS_ROWS / 4), p = e % (GS_ROWS / 4), r = ch * GS_ROWS + 4 * p;
+        const int bytes = c < k ? 4 * min(max(m - r, 0), 4) : 0;  // the rest is zero
+        cp_async16_part(&D[c][4 * (p ^ ((c >> 2) & 7))], bytes ? Lt + c * lda + r : Lt, bytes);
       }
     }
+    cp_async_commit();
+  };
+  float acc[4][4] = {};
+  stage(0);
+  stage(1);
+  for (int ch = 0; ch < chunks; ++ch) {
+    cp_async_wait<1>();
+    __syncthreads();  // chunk ch is in place, and chunk ch - 1's slot is free
+    stage(ch + 2);
+    if (ti >= nt) continue;
+    const float(*D)[GS_ROWS] = S[ch % GS_STAGES];
+#pragma unroll 2
+    for (int p = 0; p < GS_ROWS / 4; ++p) {
+      float4 a[4], b[4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        a[x] = *reinterpret_cast<const float4*>(&D[4 * ti + x][4 * (p ^ (ti & 7))]);
+        b[x] = *reinterpret_cast<const float4*>(&D[4 * tj + x][4 * (p ^ (tj & 7))]);
+      }
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+          acc[x][y] = fmaf(a[x].x, b[y].x, acc[x][y]);
+          acc[x][y] = fmaf(a[x].y, b[y].y, acc[x][y]);
+          acc[x][y] = fmaf(a[x].z, b[y].z, acc[x][y]);
+          acc[x][y] = fmaf(a[x].w, b[y].w, acc[x][y]);
+        }
+    }
   }
-  if (!active) return;
+  cp_async_wait<0>();
+  if (ti >= nt) return;
   double* M = static_cast<double*>(g.C);
 #pragma unroll
   for (int x = 0; x < 4; ++x)
 #pragma unroll
     for (int y = 0; y < 4; ++y) {
       const int i = 4 * ti + x, jj = 4 * tj + y;
-      if (i < k && jj < k) M[(int64_t)i * g.ldc + jj] = (double)acc[x][y];
+      if (i >= k || jj >= k) continue;
+      M[(int64_t)i * g.ldc + jj] = (double)acc[x][y];
+      if (ti != tj) M[(int64_t)jj * g.ldc + i] = (double)acc[x][y];
     }
 }
 
 int32_t gram_small_batched(const GemmArgs* jobs_dev, int count, cudaStream_t s) {
   if (count <= 0) return RLU_OK;
-  k_gram_small_batched<<<(unsigned)count, 256, 0, s>>>(jobs_dev);
+  k_gram_small_batched<<<(unsigned)count, GS_NT, 0, s>>>(jobs_dev);
   return last_launch_status();
 }
 
@@ -1434,30 +1474,54 @@ int32_t ldl32_batched(const Ldl32Job* jobs_dev, int count, int max_k, cudaStream
   return last_launch_status();
 }
 
+__host__ __device__ __forceinline__ int trsm_small_bucket_of(int k) {
+  return k <= 16 ? 0 : k <= 32 ? 1 : k <= 48 ? 2 : 3;
+}
+int trsm_small_bucket(int k) { return trsm_small_bucket_of(k); }
+
 // Batched form for k <= 64: one thread per column of C over a tile list of (problem,
 // 128-column block) entries. L (unit lower, from LR) sits in shared memory, zero-padded to
 // the problem's bucket KB in {16, 32, 48, 64} (padded rows and columns change nothing), and
 // the column in registers: forward substitution x_i -= sum_{j<i} L[i][j] x_j, scaling by
-// 1/D, backward substitution x_i -= sum_{j>i} L[j][i] x_j. The bucket is chosen per CTA from
-// its problem's k, so small problems do not pay for the largest k of the batch.
+// 1/D, backward substitution x_i -= sum_{j>i} L[j][i] x_j. L is held by rows and by columns, so
+// that both directions read four entries of it at a time, and the terms past k are not tested
+// for: they are products of zeros (rows past k are skipped, so that x stays zero there also
+// beside infinities). The bucket is chosen per CTA from its problem's k, so small problems do
+// not pay for the largest k of the batch; the tiles of the larger k come first. Bound by the
+// latency of one chain of k^2 multiply-adds per column: 79 us for 512 problems of n <= 1024,
+// k <= 64, 118 with a launch per bucket and L read one entry at a time backward.
 static constexpr int TS_KMAX = 64;
 static constexpr int TS_LD = TS_KMAX + 4;  // 16-byte rows
 static constexpr int TS_COLS = 128;
 
 template <int KB>
-__device__ __forceinline__ void trsm_small_body(const float (*Ls)[TS_LD], const float* dv,
-                                                const float* __restrict__ C, int64_t ldc,
-                                                float* __restrict__ B, int64_t ldb, int k,
-                                                int64_t c) {
+__device__ __forceinline__ void trsm_small_body(float (*Ls)[TS_LD], float (*Lc)[TS_LD], float* dv,
+                                                const TrsmJob& jb, int64_t c) {
+  const int k = jb.o.k, kp = jb.o.kp;
+  for (int e = threadIdx.x; e < KB * KB; e += TS_COLS) {
+    const int i = e / KB, j = e % KB;
+    const bool in = i < k && j < k;
+    Ls[i][j] = in ? jb.o.LR[(int64_t)i * kp + j] : 0.f;  // row i
+    Lc[i][j] = in ? jb.o.LT[(int64_t)i * kp + j] : 0.f;  // column i
+  }
+  for (int i = threadIdx.x; i < KB; i += TS_COLS) dv[i] = i < k ? (float)jb.o.dinv[i] : 0.f;
+  __syncthreads();
+  if (c >= jb.n) return;
   float x[KB];
 #pragma unroll
-  for (int i = 0; i < KB; ++i) x[i] = i < k ? C[(int64_t)i * ldc + c] : 0.f;
+  for (int i = 0; i < KB; ++i) x[i] = i < k ? jb.C[(int64_t)i * jb.ldc + c] : 0.f;
 #pragma unroll
   for (int i = 1; i < KB; ++i) {
     if (i < k) {
       float acc = x[i];
 #pragma unroll
-      for (int j = 0; j < i; ++j) acc = fmaf(-Ls[i][j], x[j], acc);
+      for (int j = 0; j < i; j += 4) {
+        const float4 l = *reinterpret_cast<const float4*>(&Ls[i][j]);
+        acc = fmaf(-l.x, x[j], acc);
+        if (j + 1 < i) acc = fmaf(-l.y, x[j + 1], acc);
+        if (j + 2 < i) acc = fmaf(-l.z, x[j + 2], acc);
+        if (j + 3 < i) acc = fmaf(-l.w, x[j + 3], acc);
+      }
       x[i] = acc;
     }
   }
@@ -1468,107 +1532,106 @@ __device__ __forceinline__ void trsm_small_body(const float (*Ls)[TS_LD], const 
     if (i < k - 1) {
       float acc = x[i];
 #pragma unroll
-      for (int j = i + 1; j < KB; ++j)
-        if (j < k) acc = fmaf(-Ls[j][i], x[j], acc);
+      for (int j = (i + 1) / 4 * 4; j < KB; j += 4) {
+        const float4 l = *reinterpret_cast<const float4*>(&Lc[i][j]);
+        if (j > i) acc = fmaf(-l.x, x[j], acc);
+        if (j + 1 > i) acc = fmaf(-l.y, x[j + 1], acc);
+        if (j + 2 > i) acc = fmaf(-l.z, x[j + 2], acc);
+        acc = fmaf(-l.w, x[j + 3], acc);
+      }
       x[i] = acc;
     }
   }
 #pragma unroll
   for (int i = 0; i < KB; ++i)
-    if (i < k) B[(int64_t)i * ldb + c] = x[i];
+    if (i < k) jb.B[(int64_t)i * jb.ldb + c] = x[i];
 }
 
-template <int KB>
 __global__ void __launch_bounds__(TS_COLS) k_trsm_small_batched(const TrsmJob* __restrict__ jobs,
                                                                 const int2* __restrict__ tiles) {
-  __shared__ __align__(16) float Ls[TS_KMAX][TS_LD];
+  __shared__ __align__(16) float Ls[TS_KMAX][TS_LD], Lc[TS_KMAX][TS_LD];
   __shared__ float dv[TS_KMAX];
   const int2 t = tiles[blockIdx.x];
   const TrsmJob& jb = jobs[t.x];
-  const int k = jb.o.k, kp = jb.o.kp;
-  for (int e = threadIdx.x; e < KB * KB; e += TS_COLS) {
-    const int i = e / KB, j = e % KB;
-    Ls[i][j] = (i < k && j < k) ? jb.o.LR[(int64_t)i * kp + j] : 0.f;
-  }
-  for (int i = threadIdx.x; i < KB; i += TS_COLS) dv[i] = i < k ? (float)jb.o.dinv[i] : 0.f;
-  __syncthreads();
   const int64_t c = (int64_t)t.y * TS_COLS + threadIdx.x;
-  if (c >= jb.n) return;
-  trsm_small_body<KB>(Ls, dv, jb.C, jb.ldc, jb.B, jb.ldb, k, c);
+  switch (trsm_small_bucket_of(jb.o.k)) {
+    case 0: return trsm_small_body<16>(Ls, Lc, dv, jb, c);
+    case 1: return trsm_small_body<32>(Ls, Lc, dv, jb, c);
+    case 2: return trsm_small_body<48>(Ls, Lc, dv, jb, c);
+    default: return trsm_small_body<64>(Ls, Lc, dv, jb, c);
+  }
 }
 
-int trsm_small_bucket(int k) { return k <= 16 ? 0 : k <= 32 ? 1 : k <= 48 ? 2 : 3; }
-
-int32_t trsm_small_batched(const TrsmJob* jobs_dev, const int2* tiles_dev, const int* first,
-                           const int* count, cudaStream_t s) {
-  int launches = 0;
-  for (int bkt = 0; bkt < 4; ++bkt) {
-    if (count[bkt] <= 0) continue;
-    const int2* tl = tiles_dev + first[bkt];
-    const unsigned g = (unsigned)count[bkt];
-    if (bkt == 0) k_trsm_small_batched<16><<<g, TS_COLS, 0, s>>>(jobs_dev, tl);
-    else if (bkt == 1) k_trsm_small_batched<32><<<g, TS_COLS, 0, s>>>(jobs_dev, tl);
-    else if (bkt == 2) k_trsm_small_batched<48><<<g, TS_COLS, 0, s>>>(jobs_dev, tl);
-    else k_trsm_small_batched<64><<<g, TS_COLS, 0, s>>>(jobs_dev, tl);
-    ++launches;
-  }
-  return launches ? last_launch_status(launches) : RLU_OK;
+int32_t trsm_small_batched(const TrsmJob* jobs_dev, const int2* tiles_dev, int ntiles,
+                           cudaStream_t s) {
+  if (ntiles <= 0) return RLU_OK;
+  k_trsm_small_batched<<<(unsigned)ntiles, TS_COLS, 0, s>>>(jobs_dev, tiles_dev);
+  return last_launch_status();
 }
 
 // L (m x k, column-major) = L_y (m x k, column-major, pivot order) L_b (k x k, column-major,
-// unit lower) for k <= 64: one thread per row over a tile list of (problem, 256-row block)
-// entries, L_b (zero-padded to the problem's bucket KB) in shared memory, the row of L_y in
-// registers.
+// unit lower) for k <= 64: two rows per thread (row i and i + 128 of a 256-row tile) over a
+// tile list of (problem, 256-row block) entries, L_b (zero-padded to the problem's bucket KB)
+// in shared memory, the rows of L_y in registers: 60 us for 512 problems of m <= 2048, k <= 64.
+// One row per thread was bound by the reads of L_b, a 16-byte load for four multiply-adds: 75.
 static constexpr int LM_ROWS = 256;
+static constexpr int LM_NT = LM_ROWS / 2;
 
 template <int KB>
-__device__ __forceinline__ void lmul_body(const float* Lbs, const float* __restrict__ Ly,
-                                          int64_t lda, float* __restrict__ L, int64_t ldc,
-                                          int k, int64_t i) {
-  float y[KB];
+__device__ __forceinline__ void lmul_body(const float* Lbs, const GemmArgs& g, int64_t i) {
+  const int k = (int)g.N;
+  const float* Ly = static_cast<const float*>(g.A);
+  float* L = static_cast<float*>(g.C);
+  const bool in0 = i < g.M, in1 = i + LM_NT < g.M;
+  float y0[KB], y1[KB];
 #pragma unroll
-  for (int c = 0; c < KB; ++c) y[c] = c < k ? Ly[(int64_t)c * lda + i] : 0.f;
+  for (int c = 0; c < KB; ++c) {
+    y0[c] = c < k && in0 ? Ly[(int64_t)c * g.lda + i] : 0.f;
+    y1[c] = c < k && in1 ? Ly[(int64_t)c * g.lda + i + LM_NT] : 0.f;
+  }
   for (int j = 0; j < k; ++j) {
     const float* bcol = Lbs + j * TS_LD;  // column j of L_b
-    float acc = 0.f;
+    float acc0 = 0.f, acc1 = 0.f;
 #pragma unroll
     for (int c = 0; c < KB; c += 4) {
       const float4 b4 = *reinterpret_cast<const float4*>(bcol + c);
-      acc = fmaf(y[c], b4.x, acc);
-      acc = fmaf(y[c + 1], b4.y, acc);
-      acc = fmaf(y[c + 2], b4.z, acc);
-      acc = fmaf(y[c + 3], b4.w, acc);
+      acc0 = fmaf(y0[c], b4.x, acc0);
+      acc1 = fmaf(y1[c], b4.x, acc1);
+      acc0 = fmaf(y0[c + 1], b4.y, acc0);
+      acc1 = fmaf(y1[c + 1], b4.y, acc1);
+      acc0 = fmaf(y0[c + 2], b4.z, acc0);
+      acc1 = fmaf(y1[c + 2], b4.z, acc1);
+      acc0 = fmaf(y0[c + 3], b4.w, acc0);
+      acc1 = fmaf(y1[c + 3], b4.w, acc1);
     }
-    L[(int64_t)j * ldc + i] = acc;
+    if (in0) L[(int64_t)j * g.ldc + i] = acc0;
+    if (in1) L[(int64_t)j * g.ldc + i + LM_NT] = acc1;
   }
 }
 
-__global__ void __launch_bounds__(LM_ROWS) k_lmul_batched(const GemmArgs* __restrict__ jobs,
-                                                          const int2* __restrict__ tiles) {
+__global__ void __launch_bounds__(LM_NT) k_lmul_batched(const GemmArgs* __restrict__ jobs,
+                                                        const int2* __restrict__ tiles) {
   __shared__ __align__(16) float Lbs[TS_KMAX * TS_LD];
   const int2 t = tiles[blockIdx.x];
   const GemmArgs& g = jobs[t.x];
   const int k = (int)g.N;
-  const int kb = k <= 16 ? 16 : k <= 32 ? 32 : k <= 48 ? 48 : 64;
+  const int kb = 16 * (trsm_small_bucket_of(k) + 1);
   const float* Lb = static_cast<const float*>(g.B);
-  for (int e = threadIdx.x; e < k * kb; e += LM_ROWS) {
+  for (int e = threadIdx.x; e < k * kb; e += LM_NT) {
     const int j = e / kb, c = e % kb;  // column j, entry c
     Lbs[j * TS_LD + c] = c < k ? Lb[(int64_t)j * g.ldb + c] : 0.f;
   }
   __syncthreads();
   const int64_t i = (int64_t)t.y * LM_ROWS + threadIdx.x;
-  if (i >= g.M) return;
-  const float* Ly = static_cast<const float*>(g.A);
-  float* L = static_cast<float*>(g.C);
-  if (kb == 16) lmul_body<16>(Lbs, Ly, g.lda, L, g.ldc, k, i);
-  else if (kb == 32) lmul_body<32>(Lbs, Ly, g.lda, L, g.ldc, k, i);
-  else if (kb == 48) lmul_body<48>(Lbs, Ly, g.lda, L, g.ldc, k, i);
-  else lmul_body<64>(Lbs, Ly, g.lda, L, g.ldc, k, i);
+  if (kb == 16) lmul_body<16>(Lbs, g, i);
+  else if (kb == 32) lmul_body<32>(Lbs, g, i);
+  else if (kb == 48) lmul_body<48>(Lbs, g, i);
+  else lmul_body<64>(Lbs, g, i);
 }
 
 int32_t lmul_batched(const GemmArgs* jobs_dev, const int2* tiles_dev, int ntiles, cudaStream_t s) {
   if (ntiles <= 0) return RLU_OK;
-  k_lmul_batched<<<(unsigned)ntiles, LM_ROWS, 0, s>>>(jobs_dev, tiles_dev);
+  k_lmul_batched<<<(unsigned)ntiles, LM_NT, 0, s>>>(jobs_dev, tiles_dev);
   return last_launch_status();
 }
 
@@ -1587,18 +1650,36 @@ int32_t trsm_batched(const TrsmJob* jobs_dev, const int2* tiles_dev, int ntiles,
   return last_launch_status();
 }
 
-// One CTA per problem: U (k rows of n) and L_b (k x k) in loops.
-__global__ void k_gather_batched(const GatherJob* __restrict__ jobs) {
+// CTA (problem blockIdx.x, group blockIdx.y) of U (k x n) and L_b (k x k): BG rows of B at a
+// time, staged in shared memory and read from there at the pivot columns (a column Q outside
+// [0, n), of an LU that stopped early, reads zero). 21 us for 512 problems of n <= 1024,
+// k <= 64; one CTA per problem that gathered from memory took 96.
+template <int BG>
+__global__ void __launch_bounds__(256) k_gather_batched(const GatherJob* __restrict__ jobs) {
+  extern __shared__ float gb_row[];  // [BG][n]
   const GatherJob& j = jobs[blockIdx.x];
-  const int k = j.k;
-  const int64_t n = j.n;
-  for (int i = 0; i < k; ++i) {
-#pragma unroll 4
-    for (int64_t c = threadIdx.x; c < n; c += blockDim.x)
-      j.U[(int64_t)i * j.ldu + c] = c >= i ? j.B[(int64_t)i * j.ldb + j.Q[c]] : 0.f;
-    // L_b column i: rows r > i from B's row r at the pivot column Q[i]
-    for (int r = threadIdx.x; r < k; r += blockDim.x)
-      j.Lb[(int64_t)i * k + r] = r > i ? j.B[(int64_t)r * j.ldb + j.Q[i]] : (r == i ? 1.f : 0.f);
+  const int n = (int)j.n, k = j.k;
+  for (int i0 = BG * blockIdx.y; i0 < k; i0 += BG * gridDim.y) {
+    for (int c = threadIdx.x; c < n; c += blockDim.x) {
+      float v[BG];
+#pragma unroll
+      for (int u = 0; u < BG; ++u) v[u] = i0 + u < k ? j.B[(int64_t)(i0 + u) * j.ldb + c] : 0.f;
+#pragma unroll
+      for (int u = 0; u < BG; ++u) gb_row[u * n + c] = v[u];
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < n; c += blockDim.x) {
+      const int q = j.Q[c];
+      const bool in = q >= 0 && q < n;
+#pragma unroll
+      for (int u = 0; u < BG; ++u) {
+        const float v = in ? gb_row[u * n + q] : 0.f;
+        if (i0 + u < k) j.U[(int64_t)(i0 + u) * j.ldu + c] = c >= i0 + u ? v : 0.f;
+        if (c < k && i0 + u < k)  // L_b column c: rows r > c from B's row r at column Q[c]
+          j.Lb[(int64_t)c * k + i0 + u] = i0 + u > c ? v : (i0 + u == c ? 1.f : 0.f);
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -1606,8 +1687,12 @@ int32_t gather_batched(const GatherJob* jobs_dev, int count, int max_k, int64_t 
                        cudaStream_t s) {
   if (count <= 0) return RLU_OK;
   (void)max_k;
-  (void)max_n;
-  k_gather_batched<<<(unsigned)count, 256, 0, s>>>(jobs_dev);
+  const bool four = max_n <= BG_LONG;
+  const auto kernel = four ? k_gather_batched<4> : k_gather_batched<1>;
+  const size_t smem = (size_t)max_n * sizeof(float) * (four ? 4 : 1);
+  RLU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem));
+  kernel<<<dim3((unsigned)count, 8), 256, smem, s>>>(jobs_dev);
   return last_launch_status();
 }
 
