@@ -174,7 +174,7 @@ struct rlu_batch {
   // LU groups: 1..16 = clusters of that many CTAs of lu_rows_per_cta rows; 17 / 18 = one CTA
   // of 128 / 256 threads for problems of at most 128 / 256 rows
   int first_y[rlu::kLuGroups] = {}, count_y[rlu::kLuGroups] = {}, first_b[rlu::kLuGroups] = {},
-      count_b[rlu::kLuGroups] = {};
+      count_b[rlu::kLuGroups] = {}, wide_y[rlu::kLuGroups] = {}, wide_b[rlu::kLuGroups] = {};
   int launches = 0;
   // tensor-core rings of the mixed precision (Y = A G, C = L~^T A)
   int u3y_stages = 0, u3y_stage_bytes = 0, u3c_stages = 0, u3c_stage_bytes = 0;
@@ -370,7 +370,7 @@ extern "C" int32_t rlu_batch_create(const rlu_problem* problems, int32_t count, 
                    [](const GemmArgs& x, const GemmArgs& y) { return x.K > y.K; });
   // LU records grouped by cluster size
   auto group = [&](const std::vector<LuArgs>& all, const std::vector<int>& gof, int* first,
-                   int* cnt, std::vector<LuArgs>& sorted) {
+                   int* cnt, int* wide, std::vector<LuArgs>& sorted) {
     for (int g = 0; g < kLuGroups; ++g) cnt[g] = 0;
     for (int v : gof) ++cnt[v];
     int acc = 0;
@@ -381,10 +381,20 @@ extern "C" int32_t rlu_batch_create(const rlu_problem* problems, int32_t count, 
     std::vector<int> fill(first, first + kLuGroups);
     sorted.resize(all.size());
     for (size_t i = 0; i < all.size(); ++i) sorted[(size_t)fill[gof[i]]++] = all[i];
+    for (int g = 0; g < kLuGroups; ++g) {  // an LU's time is its columns: the longest first
+      const auto at = sorted.begin() + first[g];
+      std::stable_sort(at, at + cnt[g],
+                       [](const LuArgs& x, const LuArgs& y) { return x.C > y.C; });
+      // CTAs of up to 256 rows share an SM at any width: one launch
+      const bool split = g >= 1 && g <= 16 && opt.lu_rows_per_cta == 512;
+      wide[g] = split ? (int)std::count_if(at, at + cnt[g],
+                                           [](const LuArgs& x) { return x.C > kLuNarrow; })
+                      : cnt[g];
+    }
   };
   std::vector<LuArgs> luy, lub;
-  group(luy_all, gy_of, b->first_y, b->count_y, luy);
-  group(lub_all, gb_of, b->first_b, b->count_b, lub);
+  group(luy_all, gy_of, b->first_y, b->count_y, b->wide_y, luy);
+  group(lub_all, gb_of, b->first_b, b->count_b, b->wide_b, lub);
 
   auto up = [&](size_t off, const void* src, size_t bytes) -> int32_t {
     RLU_CUDA_TRY(cudaMemcpy(ws + off, src, bytes, cudaMemcpyHostToDevice));
@@ -438,14 +448,22 @@ extern "C" int32_t rlu_batch_create(const rlu_problem* problems, int32_t count, 
     b->u3c_stage_bytes = max_stage_c;
     if (st == RLU_OK) st = up(t.u3y, u3y.data(), c * sizeof(U3Job));
     if (st == RLU_OK) st = up(t.u3c, u3c.data(), c * sizeof(U3Job));
-    // tile lists: the tiles of one problem next to each other
+    // tile lists: the tiles of one problem next to each other, the problems with the longest
+    // tiles first (a CTA takes the next tile when it is done with one; C's 128-row tiles over
+    // m <= 2048 157 -> 141 us, Y's unchanged)
     std::vector<int2> ty, tc;
     ty.reserve((size_t)t.n_tiles_y);
     tc.reserve((size_t)t.n_tiles_c);
-    for (int i = 0; i < count; ++i) {
+    std::vector<int> order((size_t)count);
+    for (int i = 0; i < count; ++i) order[(size_t)i] = i;
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int x, int y) { return problems[x].n > problems[y].n; });
+    for (int i : order)
       for (int mt = 0; mt < (int)ceil_div(problems[i].m, 128); ++mt) ty.push_back(make_int2(i, mt));
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int x, int y) { return problems[x].m > problems[y].m; });
+    for (int i : order)
       for (int mt = 0; mt < (int)ceil_div(problems[i].n, 128); ++mt) tc.push_back(make_int2(i, mt));
-    }
     if (st == RLU_OK) st = up(t.u3y_tiles, ty.data(), ty.size() * sizeof(int2));
     if (st == RLU_OK) st = up(t.u3c_tiles, tc.data(), tc.size() * sizeof(int2));
   }
@@ -454,7 +472,9 @@ extern "C" int32_t rlu_batch_create(const rlu_problem* problems, int32_t count, 
     return st;
   }
   int groups = 0;
-  for (int g = 1; g < kLuGroups; ++g) groups += (b->count_y[g] > 0) + (b->count_b[g] > 0);
+  for (int g = 1; g < kLuGroups; ++g)
+    groups += (b->wide_y[g] > 0) + (b->count_y[g] > b->wide_y[g]) + (b->wide_b[g] > 0) +
+              (b->count_b[g] > b->wide_b[g]);
   b->launches = 10 + groups;
   *out = b;
   return RLU_OK;
@@ -483,7 +503,7 @@ extern "C" int32_t rlu_factor_batched(rlu_batch* b, void* stream) {
                                              b->opt.gemm_tile_y)));
   RLU_TRY(launch_lu_reg_batched(false, b->opt.lu_rows_per_cta,
                                 reinterpret_cast<const LuArgs*>(ws + t.lu_y), b->first_y,
-                                b->count_y, s, b->have_fork ? &b->lu_fork : nullptr));
+                                b->count_y, b->wide_y, s, b->have_fork ? &b->lu_fork : nullptr));
   RLU_TRY(build_ly_batched(reinterpret_cast<const BuildJob*>(ws + t.build), c, b->max_m,
                            b->max_k, s));
   if (t.small_k)  // the Gram is k x k with k <= 64: one CTA per problem
@@ -511,7 +531,7 @@ extern "C" int32_t rlu_factor_batched(rlu_batch* b, void* stream) {
                          s));
   RLU_TRY(launch_lu_reg_batched(true, b->opt.lu_rows_per_cta,
                                 reinterpret_cast<const LuArgs*>(ws + t.lu_b), b->first_b,
-                                b->count_b, s, b->have_fork ? &b->lu_fork : nullptr));
+                                b->count_b, b->wide_b, s, b->have_fork ? &b->lu_fork : nullptr));
   RLU_TRY(gather_batched(reinterpret_cast<const GatherJob*>(ws + t.gather), c, b->max_k,
                          b->max_n, s));
   if (t.small_k)

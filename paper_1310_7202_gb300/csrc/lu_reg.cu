@@ -1023,7 +1023,7 @@ __global__ void __launch_bounds__(NC + kLuUpd, 1) k_lu_reg(LuArgs a) {
 
 // Batched form: cluster c of the launch factors problem table[c] (one panel: pw = C).
 template <typename T, bool CROUT, int RT, int NC, bool SOLO>
-__global__ void __launch_bounds__(NC + kLuUpd, 1) k_lu_reg_batched(const LuArgs* __restrict__ table,
+__global__ void __launch_bounds__(NC + kLuUpd, 2) k_lu_reg_batched(const LuArgs* __restrict__ table,
                                                                    int pw) {
   const int csize = (int)cg::this_cluster().num_blocks();
   LuArgs a = table[blockIdx.x / csize];
@@ -1277,8 +1277,12 @@ int32_t launch_lu_reg(int32_t dtype, bool crout, const LuArgs& a, cudaStream_t s
 // Batched LUs of problems that fit one register panel (C <= NB - 1 = 76 FP32 columns, R <=
 // 16 x rows_per_cta): the table on the device is grouped by cluster size (ceil(R /
 // rows_per_cta) CTAs); group g starts at table entry first[g] and holds count[g] problems.
-// rows_per_cta is 512 (512-thread CTAs) or 256 (256-thread CTAs, twice as many CTAs per
-// problem).
+// rows_per_cta is 512 or 256 (twice as many CTAs per problem). A panel of 76 columns of 512 rows
+// takes more than half an SM's shared memory, and a step of one CTA leaves its SM idle while it
+// waits; the groups of 512-row CTAs are therefore launched in two parts, up to 48 columns (108 KB
+// a CTA) and more, and no CTA takes more than 128 registers a thread, so that two share an SM.
+// With the longest LUs of a group first, 512 problems (m <= 2048, k <= 64) 1239 -> 1168 us, of
+// which 16 us are the order of the C product's tiles.
 template <int RT>
 static int32_t lu_batched_group(bool crout, const LuArgs* table_dev, int first, int count, int g,
                                 int pw, cudaStream_t s) {
@@ -1313,34 +1317,39 @@ static int32_t lu_batched_group(bool crout, const LuArgs* table_dev, int first, 
 }
 
 int32_t launch_lu_reg_batched(bool crout, int rows_per_cta, const LuArgs* table_dev,
-                              const int* first, const int* count, cudaStream_t s,
-                              const LuFork* fork) {
+                              const int* first, const int* count, const int* wide,
+                              cudaStream_t s, const LuFork* fork) {
   if (rows_per_cta != 512 && rows_per_cta != 256) return RLU_EINVAL;
-  int groups[kLuGroups], ng = 0;
-  for (int g = 16; g >= 1; --g)  // widest clusters first
-    if (count[g] > 0) groups[ng++] = g;
-  for (int g : {17, 18})  // one narrow CTA for small problems, several per SM
-    if (count[g] > 0) groups[ng++] = g;
-  const bool par = fork != nullptr && ng > 1;
+  struct Part {
+    int g, first, count, pw;
+  } parts[2 * kLuGroups];
+  int np = 0;
+  auto add = [&](int g) {
+    if (wide[g] > 0) parts[np++] = {g, first[g], wide[g], 76};
+    if (count[g] > wide[g]) parts[np++] = {g, first[g] + wide[g], count[g] - wide[g], kLuNarrow};
+  };
+  for (int g = 16; g >= 1; --g) add(g);  // widest clusters first
+  for (int g : {17, 18}) add(g);         // one CTA for small problems, several per SM
+  const bool par = fork != nullptr && np > 1;
   if (par) RLU_CUDA_TRY(cudaEventRecord(fork->fork, s));
-  for (int i = 0; i < ng; ++i) {
-    const int g = groups[i];
+  for (int i = 0; i < np; ++i) {
+    const Part& p = parts[i];
     cudaStream_t gs = s;
     if (par) {
       gs = fork->hs[i % kLuSide];
       if (i < kLuSide) RLU_CUDA_TRY(cudaStreamWaitEvent(gs, fork->fork, 0));
     }
-    if (g == 17)
-      RLU_TRY(lu_batched_group<1>(crout, table_dev, first[g], count[g], 1, 76, gs));
-    else if (g == 18)
-      RLU_TRY(lu_batched_group<2>(crout, table_dev, first[g], count[g], 1, 76, gs));
+    if (p.g == 17)
+      RLU_TRY(lu_batched_group<1>(crout, table_dev, p.first, p.count, 1, p.pw, gs));
+    else if (p.g == 18)
+      RLU_TRY(lu_batched_group<2>(crout, table_dev, p.first, p.count, 1, p.pw, gs));
     else if (rows_per_cta == 512)
-      RLU_TRY(lu_batched_group<4>(crout, table_dev, first[g], count[g], g, 76, gs));
+      RLU_TRY(lu_batched_group<4>(crout, table_dev, p.first, p.count, p.g, p.pw, gs));
     else
-      RLU_TRY(lu_batched_group<2>(crout, table_dev, first[g], count[g], g, 76, gs));
+      RLU_TRY(lu_batched_group<2>(crout, table_dev, p.first, p.count, p.g, p.pw, gs));
   }
   if (par)
-    for (int i = 0; i < ng && i < kLuSide; ++i) {
+    for (int i = 0; i < np && i < kLuSide; ++i) {
       RLU_CUDA_TRY(cudaEventRecord(fork->join[i], fork->hs[i]));
       RLU_CUDA_TRY(cudaStreamWaitEvent(s, fork->join[i], 0));
     }

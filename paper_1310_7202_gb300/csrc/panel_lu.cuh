@@ -49,14 +49,17 @@ static constexpr int kLuGroups = 19;
 // its own helper stream (fork / join events around them on s), so that the groups' CTAs
 // share the GPU instead of running one launch after another; works under stream capture
 // (parallel branches of the graph).
-static constexpr int kLuSide = 6;
+static constexpr int kLuSide = 12;
+// wide[g] of a group's entries, its first ones, have more than kLuNarrow columns; the rest are
+// launched by themselves, with shared memory for that many, so that two CTAs share an SM.
+static constexpr int kLuNarrow = 48;
 struct LuFork {
   cudaStream_t hs[kLuSide];
   cudaEvent_t fork;
   cudaEvent_t join[kLuSide];
 };
 int32_t launch_lu_reg_batched(bool crout, int rows_per_cta, const LuArgs* table_dev,
-                              const int* first, const int* count, cudaStream_t s,
-                              const LuFork* fork = nullptr);
+                              const int* first, const int* count, const int* wide,
+                              cudaStream_t s, const LuFork* fork = nullptr);
 
 }  // namespace rlu

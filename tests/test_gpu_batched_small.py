@@ -1,6 +1,6 @@
 """The batch's kernels for k <= 64 at the edges of their tiles: buckets of k (16, 32, 48, 64),
-4 x 4 blocks of the Gram, 64-row chunks, 256-row and 128-column blocks, and batches whose
-longest side passes 2048 (one staged column instead of four). Each problem is compared with
+4 x 4 blocks of the Gram, 64-row chunks, 256-row and 128-column blocks, LUs of 48 and 49
+columns, and batches whose longest side passes 2048 (one staged column instead of four). Each problem is compared with
 the single-problem path, which uses none of these kernels. Both round in FP32, so the error of
 the batch's factors stays within 1.1 of the other's plus 1e-4 ||A||_2, the tolerance of the
 batch's other tests; a wrong row, column or chunk leaves an error of the order of ||A||. GPU only."""
@@ -20,7 +20,9 @@ SHORT = [(64, 64, 1), (65, 64, 4), (127, 65, 15), (128, 127, 16), (129, 128, 17)
 
 @pytest.mark.parametrize("prec", ["f32", "mixed"])
 @pytest.mark.parametrize("extra", [[], [(2048, 200, 21)], [(2051, 90, 40), (100, 90, 7)],
-                                   [(2100, 2053, 64)]])
+                                   [(2100, 2053, 64)],
+                                   # LUs of 48 columns and of 49, launched apart
+                                   [(600, 560, 38), (601, 550, 39), (300, 280, 48)]])
 def test_edges_of_the_small_kernels(prec, extra):
     mats, probs = [], []
     for i, (m, n, k) in enumerate(SHORT + extra):
