@@ -1027,19 +1027,68 @@ __global__ void __launch_bounds__(TB / 2 * 64 / 4) k_trsm_batched(const TrsmJob*
 // work in flight. A pass needs 32 contiguous rows of L^T (forward: L^T row 32 J + t, columns
 // past the block) or of L (backward: L row 32 J + t, columns before the block) and the
 // diagonal block's inverse (W_J, or W_J^T backward): they stream into the other slot of a
-// two-slot cp.async ring while the current pass computes. 256 threads; in the update passes
+// two-slot cp.async ring while the current pass computes. In the update passes
 // each thread owns a TR x 4 tile (a warp: 32 / (TC / 4) row groups x TC / 4 column groups),
 // so every k-step is TR / 4 + 1 16-byte shared loads for 4 TR multiply-adds. D^{-1} is
 // applied in the storage precision (its reciprocals rounded once).
-static constexpr int RL_NT = 256;
+// FP32 takes 512 threads (one CTA per SM fits for k > 150, and with 8 warps a pass over more
+// than 8 strips took two rounds) and its update passes two rows to an instruction
+// (fma.rn.f32x2, the same rounding; with three different registers per multiply-add the scalar
+// form reaches 164 of 250 G/s per SM): k = 512, n = 16384 471 -> 448 us, k = 200, n = 8192
+// 51 -> 49. A pass over few strips is bound by one strip's chain, not by the rate: up to half as
+// many strips as warps are taken half as high: 406 us and 47.
+template <typename T>
+constexpr int RL_NT = sizeof(T) == 4 ? 512 : 256;
+
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(v));
+  return d;
+}
+// acc (TR x 4, rows in pairs) += l x^T over TB rows t of l (row stride LP) and x (row stride TC)
+template <int TC, int TR>
+__device__ __forceinline__ void rl_update(const float* l, const float* x, int LP,
+                                          float (&acc)[TR][4]) {
+  uint64_t p[TR / 2][4] = {};
+#pragma unroll 4
+  for (int t = 0; t < TB; ++t) {
+    const float4 xv = *reinterpret_cast<const float4*>(x + t * TC);
+    const uint64_t xx[4] = {pack2(xv.x, xv.x), pack2(xv.y, xv.y), pack2(xv.z, xv.z),
+                            pack2(xv.w, xv.w)};
+#pragma unroll
+    for (int h = 0; h < TR / 4; ++h) {
+      const ulonglong2 lv = *reinterpret_cast<const ulonglong2*>(l + t * LP + 4 * h);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(p[2 * h][b]) : "l"((uint64_t)lv.x), "l"(xx[b]));
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(p[2 * h + 1][b]) : "l"((uint64_t)lv.y), "l"(xx[b]));
+      }
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < TR / 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const float2 v = unpack2(p[a][b]);
+      acc[2 * a][b] = v.x;
+      acc[2 * a + 1][b] = v.y;
+    }
+}
 
 template <typename T>
 __host__ __device__ constexpr int rl_lpad(int kp) { return kp + 16 / (int)sizeof(T); }
 
 template <typename T, int TC, int TR>
-__global__ void __launch_bounds__(RL_NT) k_trsm_rl(LdlOut<T> o, const T* __restrict__ C,
+__global__ void __launch_bounds__(RL_NT<T>) k_trsm_rl(LdlOut<T> o, const T* __restrict__ C,
                                                    int64_t ldc, int64_t n, T* __restrict__ B,
                                                    int64_t ldb) {
+  constexpr int NT = RL_NT<T>;
+  constexpr int DR = TB / (NT / 32);  // rows per warp in the diagonal passes
   constexpr int CH = 16 / sizeof(T);  // elements per 16-byte copy
   constexpr int CG = TC / 4;          // column groups of a warp in the update passes
   constexpr int RG = 32 / CG;         // row groups (8 rows each) of a warp
@@ -1063,13 +1112,13 @@ __global__ void __launch_bounds__(RL_NT) k_trsm_rl(LdlOut<T> o, const T* __restr
       const T* Lsrc = fwd ? o.LT : o.LR;
       T* Ld = Ls + (size_t)(q & 1) * TB * LP;
       const int per = (i1 - i0) / CH;  // 16-byte pieces per row
-      for (int e = tid; e < TB * per; e += RL_NT) {
+      for (int e = tid; e < TB * per; e += NT) {
         const int t = e / per, i = i0 + (e % per) * CH;
         cp_async16(Ld + t * LP + (i - i0), Lsrc + (int64_t)(J * TB + t) * kp + i);
       }
       const T* Wsrc = (fwd ? o.W : o.WT) + (size_t)J * TB * TB;
       T* Wd = Wsm + (size_t)(q & 1) * TB * LSP;
-      for (int e = tid; e < TB * TB / CH; e += RL_NT) {
+      for (int e = tid; e < TB * TB / CH; e += NT) {
         const int r = e / (TB / CH), c = (e % (TB / CH)) * CH;
         cp_async16(Wd + r * LSP + c, Wsrc + r * TB + c);
       }
@@ -1077,20 +1126,20 @@ __global__ void __launch_bounds__(RL_NT) k_trsm_rl(LdlOut<T> o, const T* __restr
     cp_async_commit();
   };
   stage(0);
-  for (int i = tid; i < kp; i += RL_NT) Dsm[i] = i < k ? (T)o.dinv[i] : T(0);
+  for (int i = tid; i < kp; i += NT) Dsm[i] = i < k ? (T)o.dinv[i] : T(0);
   constexpr int LDU = 8;  // batches of independent loads
-  for (int e0 = tid; e0 < kp * TC; e0 += RL_NT * LDU) {
+  for (int e0 = tid; e0 < kp * TC; e0 += NT * LDU) {
     T v[LDU];
 #pragma unroll
     for (int u = 0; u < LDU; ++u) {
-      const int e = e0 + u * RL_NT, i = e / TC, c = e % TC;
+      const int e = e0 + u * NT, i = e / TC, c = e % TC;
       v[u] = (i < k && c0 + c < n) ? C[(int64_t)i * ldc + c0 + c] : T(0);
     }
 #pragma unroll
     for (int u = 0; u < LDU; ++u)
-      if (e0 + u * RL_NT < kp * TC) Xs[e0 + u * RL_NT] = v[u];
+      if (e0 + u * NT < kp * TC) Xs[e0 + u * NT] = v[u];
   }
-  const int dr = warp * 4;          // diagonal pass: rows dr .. dr + 3 of the block
+  const int dr = warp * DR;         // diagonal pass: rows dr .. dr + DR - 1 of the block
   const int dc = lane * CPT;        //   and columns dc .. dc + CPT - 1
   const int ug = lane / CG;         // update pass: row group of this thread in the warp strip
   const int uc = (lane % CG) * 4;   //   and its 4 columns
@@ -1099,71 +1148,104 @@ __global__ void __launch_bounds__(RL_NT) k_trsm_rl(LdlOut<T> o, const T* __restr
     const int J = fwd ? q : npass - 1 - q;
     if (q == nb) {  // between the directions: X = D^{-1} X
       __syncthreads();
-      for (int e = tid; e < k * TC; e += RL_NT) Xs[e] *= Dsm[e / TC];
+      for (int e = tid; e < k * TC; e += NT) Xs[e] *= Dsm[e / TC];
     }
     cp_async_wait<0>();
     __syncthreads();  // pass q's operands and the previous pass's rows of X are in place
     stage(q + 1);     // the other slot was last read by pass q - 1
     const T* Lq = Ls + (size_t)(q & 1) * TB * LP;
     const T* Wq = Wsm + (size_t)(q & 1) * TB * LSP;
-    // diagonal pass: X_J = W X_J (W = W_J forward, W_J^T backward), 4 x CPT per thread
+    // diagonal pass: X_J = W X_J (W = W_J forward, W_J^T backward), DR x CPT per thread
     T* XJ = Xs + (size_t)J * TB * TC;
-    T d[4][CPT] = {};
+    T d[DR][CPT] = {};
     // rows and columns past k are zero and stay so: FP64, whose multiply-adds count, skips
     // them (in FP32 the variable trip counts cost more: 471 -> 549 us at k = 512)
     constexpr bool kSkip = sizeof(T) == 8;
     const int tb = kSkip ? min(TB, k - J * TB) : TB;
+    if constexpr (kSkip) {
 #pragma unroll 8
-    for (int t = 0; t < (kSkip ? (dr < tb ? tb : 0) : TB); ++t) {
-      T xv[CPT];
+      for (int t = 0; t < (dr < tb ? tb : 0); ++t) {
+        T xv[CPT];
 #pragma unroll
-      for (int b = 0; b < CPT; ++b) xv[b] = XJ[t * TC + dc + b];
+        for (int b = 0; b < CPT; ++b) xv[b] = XJ[t * TC + dc + b];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const T w = Wq[(dr + a) * LSP + t];
+        for (int a = 0; a < DR; ++a) {
+          const T w = Wq[(dr + a) * LSP + t];
 #pragma unroll
-        for (int b = 0; b < CPT; ++b) d[a][b] = fma(w, xv[b], d[a][b]);
+          for (int b = 0; b < CPT; ++b) d[a][b] = fma(w, xv[b], d[a][b]);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int t = 0; t < TB; t += 4) {
+        Vec4<T> w[DR];
+#pragma unroll
+        for (int a = 0; a < DR; ++a) w[a] = lds4(Wq + (dr + a) * LSP + t);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int b = 0; b < CPT; ++b) {
+            const T xv = XJ[(t + u) * TC + dc + b];
+#pragma unroll
+            for (int a = 0; a < DR; ++a) d[a][b] = fma(w[a].v[u], xv, d[a][b]);
+          }
       }
     }
     __syncthreads();  // every thread has read X_J
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < DR; ++a)
 #pragma unroll
       for (int b = 0; b < CPT; ++b)
         if (!kSkip || dr < tb) XJ[(dr + a) * TC + dc + b] = d[a][b];
     __syncthreads();
     // update pass: rows i0 .. i1 - 1 of X minus (staged rows t of L^T / L) x X_J
     const int i0 = fwd ? (J + 1) * TB : 0, i1 = fwd ? kp : J * TB;
-    const int strips = (i1 - i0) / (RG * TR);
-    for (int st = warp; st < strips; st += RL_NT / 32) {
-      const int r0 = st * RG * TR + ug * TR;  // row offset within the updated range
-      T acc[TR][4] = {};
+    auto update = [&](auto rows) {
+      constexpr int R = decltype(rows)::value;
+      const int strips = (i1 - i0) / (RG * R);
+      for (int st = warp; st < strips; st += NT / 32) {
+        const int r0 = st * RG * R + ug * R;  // row offset within the updated range
+        T acc[R][4] = {};
+        if constexpr (kSkip) {
 #pragma unroll 4
-      for (int t = 0; t < (kSkip ? tb : TB); ++t) {
-        const Vec4<T> x = lds4(XJ + t * TC + uc);
+          for (int t = 0; t < tb; ++t) {
+            const Vec4<T> x = lds4(XJ + t * TC + uc);
 #pragma unroll
-        for (int h = 0; h < TR / 4; ++h) {
-          const Vec4<T> l = lds4(Lq + t * LP + r0 + 4 * h);
+            for (int h = 0; h < R / 4; ++h) {
+              const Vec4<T> l = lds4(Lq + t * LP + r0 + 4 * h);
 #pragma unroll
-          for (int b = 0; b < 4; ++b)
+              for (int b = 0; b < 4; ++b)
 #pragma unroll
-            for (int a = 0; a < 4; ++a) acc[4 * h + a][b] = fma(l.v[a], x.v[b], acc[4 * h + a][b]);
+                for (int a = 0; a < 4; ++a) acc[4 * h + a][b] = fma(l.v[a], x.v[b], acc[4 * h + a][b]);
+            }
+          }
+        } else {
+          rl_update<TC, R>(Lq + r0, XJ + uc, LP, acc);
+        }
+#pragma unroll
+        for (int a = 0; a < R; ++a) {
+          T* xr = Xs + (size_t)(i0 + r0 + a) * TC + uc;
+          const Vec4<T> cur = lds4(xr);
+          if constexpr (sizeof(T) == 4) {
+            *reinterpret_cast<float4*>(xr) = make_float4(cur.v[0] - acc[a][0], cur.v[1] - acc[a][1],
+                                                         cur.v[2] - acc[a][2], cur.v[3] - acc[a][3]);
+          } else {
+#pragma unroll
+            for (int b = 0; b < 4; ++b) xr[b] = cur.v[b] - acc[a][b];
+          }
         }
       }
-#pragma unroll
-      for (int a = 0; a < TR; ++a) {
-        T* xr = Xs + (size_t)(i0 + r0 + a) * TC + uc;
-        const Vec4<T> cur = lds4(xr);
-        xr[0] = cur.v[0] - acc[a][0];
-        xr[1] = cur.v[1] - acc[a][1];
-        xr[2] = cur.v[2] - acc[a][2];
-        xr[3] = cur.v[3] - acc[a][3];
-      }
+    };
+    if constexpr (sizeof(T) == 4 && TR == 8) {  // few strips: half as high, over more warps
+      if ((i1 - i0) / (RG * 8) <= NT / 64) update(std::integral_constant<int, 4>{});
+      else update(std::integral_constant<int, 8>{});
+    } else {
+      update(std::integral_constant<int, TR>{});
     }
   }
   cp_async_wait<0>();
   __syncthreads();
-  for (int e = tid; e < k * TC; e += RL_NT) {
+  for (int e = tid; e < k * TC; e += NT) {
     const int i = e / TC, c = e % TC;
     if (c0 + c < n) B[(int64_t)i * ldb + c0 + c] = Xs[e];
   }
@@ -1181,7 +1263,7 @@ static int32_t trsm_rl_launch(const LdlOut<T>& o, const T* C, int64_t ldc, int64
   const size_t bytes = trsm_rl_smem_bytes<T>(o.kp, TC);
   RLU_CUDA_TRY(cudaFuncSetAttribute(k_trsm_rl<T, TC, TR>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  k_trsm_rl<T, TC, TR><<<(unsigned)ceil_div(n, TC), RL_NT, bytes, s>>>(o, C, ldc, n, B, ldb);
+  k_trsm_rl<T, TC, TR><<<(unsigned)ceil_div(n, TC), RL_NT<T>, bytes, s>>>(o, C, ldc, n, B, ldb);
   return last_launch_status();
 }
 
