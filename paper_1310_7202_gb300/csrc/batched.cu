@@ -365,9 +365,10 @@ extern "C" int32_t rlu_batch_create(const rlu_problem* problems, int32_t count, 
     b->max_l = std::max(b->max_l, p.l);
     b->max_kp = std::max(b->max_kp, L.kp);
   }
-  // the Gram matrices' sums run over m in order: the longest first
-  std::stable_sort(gg.begin(), gg.end(),
-                   [](const GemmArgs& x, const GemmArgs& y) { return x.K > y.K; });
+  // the Gram matrices' sums run over m in order: the largest first
+  std::stable_sort(gg.begin(), gg.end(), [](const GemmArgs& x, const GemmArgs& y) {
+    return x.K * x.N * x.N > y.K * y.N * y.N;
+  });
   // LU records grouped by cluster size
   auto group = [&](const std::vector<LuArgs>& all, const std::vector<int>& gof, int* first,
                    int* cnt, int* wide, std::vector<LuArgs>& sorted) {

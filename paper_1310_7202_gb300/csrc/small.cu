@@ -1459,27 +1459,32 @@ int32_t build_ly_batched(const BuildJob* jobs_dev, int count, int64_t max_m, int
   return last_launch_status();
 }
 
-// Gram M = L~^T L~ (k x k, FP64 out, FP32 accumulation) for k <= 64: one CTA per problem;
-// thread t holds the t-th 4 x 4 block of the lower triangle (M is symmetric to the bit: the
-// same products in the same order) and stores it on both sides. A sum runs over m in order, so
-// the longest problem's chain bounds the kernel: 64 rows of every column are staged at a time,
-// two chunks ahead of the one in use, and a step of four rows is eight 16-byte loads for 64
-// multiply-adds. The 16-byte pieces of a column are stored at their number xor column / 4, so
-// that eight neighbouring blocks read different banks. 99 us for 512 problems of m <= 2048,
-// k <= 64; full squares, 32-row chunks and one chunk ahead took 155.
+// Gram M = L~^T L~ (k x k, FP64 out, FP32 accumulation) for k <= 64: two CTAs per problem, one
+// where 32 threads do; a thread holds a 4 x 4 block of the lower triangle (M is symmetric to
+// the bit: the same products in the same order) and stores it on both sides. A sum runs over m
+// in order, so the SMs with the longest problems bound the kernel, and they by their shared
+// loads: 64 rows of every column are staged at a time, two chunks ahead of the one in use, and a
+// step of four rows is eight 16-byte loads for 64 multiply-adds. The 16-byte pieces of a column
+// are stored at their number xor column / 4, so that eight neighbouring blocks read different
+// banks. 71 us for 512 problems of m <= 2048, k <= 64; 99 with one CTA per problem, 155 with
+// full squares, 32-row chunks and one chunk ahead.
 static constexpr int GS_KMAX = 64;
 static constexpr int GS_ROWS = 64;
 static constexpr int GS_STAGES = 3;
-static constexpr int GS_NT = 160;  // 136 blocks at k = 64
+static constexpr int GS_NT = 96;  // half of the 136 blocks at k = 64
 __global__ void __launch_bounds__(GS_NT) k_gram_small_batched(const GemmArgs* __restrict__ jobs) {
   __shared__ __align__(16) float S[GS_STAGES][GS_KMAX][GS_ROWS];
-  const GemmArgs& g = jobs[blockIdx.x];
+  const GemmArgs& g = jobs[blockIdx.y];
   const int k = (int)g.N, m = (int)g.K, nt = (k + 3) / 4, tid = threadIdx.x;
   const float* Lt = static_cast<const float*>(g.A);
   const int64_t lda = g.lda;
+  const int blocks = nt * (nt + 1) / 2, half = blocks <= 32 ? blocks : (blocks + 1) / 2;
+  if ((int)blockIdx.x * half >= blocks) return;
+  const int t = (int)blockIdx.x * half + tid;
   int ti = 0;
-  while ((ti + 1) * (ti + 2) / 2 <= tid) ++ti;
-  const int tj = tid - ti * (ti + 1) / 2;
+  while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+  const int tj = t - ti * (ti + 1) / 2;
+  const bool active = tid < half && ti < nt;
   const int chunks = (m + GS_ROWS - 1) / GS_ROWS;
   auto stage = [&](int ch) {
     if (ch < chunks) {
@@ -1499,7 +1504,7 @@ __global__ void __launch_bounds__(GS_NT) k_gram_small_batched(const GemmArgs* __
     cp_async_wait<1>();
     __syncthreads();  // chunk ch is in place, and chunk ch - 1's slot is free
     stage(ch + 2);
-    if (ti >= nt) continue;
+    if (!active) continue;
     const float(*D)[GS_ROWS] = S[ch % GS_STAGES];
 #pragma unroll 2
     for (int p = 0; p < GS_ROWS / 4; ++p) {
@@ -1521,7 +1526,7 @@ __global__ void __launch_bounds__(GS_NT) k_gram_small_batched(const GemmArgs* __
     }
   }
   cp_async_wait<0>();
-  if (ti >= nt) return;
+  if (!active) return;
   double* M = static_cast<double*>(g.C);
 #pragma unroll
   for (int x = 0; x < 4; ++x)
@@ -1536,7 +1541,7 @@ __global__ void __launch_bounds__(GS_NT) k_gram_small_batched(const GemmArgs* __
 
 int32_t gram_small_batched(const GemmArgs* jobs_dev, int count, cudaStream_t s) {
   if (count <= 0) return RLU_OK;
-  k_gram_small_batched<<<(unsigned)count, GS_NT, 0, s>>>(jobs_dev);
+  k_gram_small_batched<<<dim3(2, (unsigned)count), GS_NT, 0, s>>>(jobs_dev);
   return last_launch_status();
 }
 
