@@ -712,6 +712,10 @@ __device__ __forceinline__ void lu_reg_body(const LuArgs& a) {
             for (int e = 0; e < EPC; ++e) P[1 + E0 + (q - 1) * EPC + e] = v[e];
           }
         }
+        if (timed_out) {  // the records may not have come: no pivot, positions stay as they are
+          wpr = kNone;
+          P[0] = T(0);
+        }
         if (SOLO) rp = rcp_piv(P[0]);
         const bool nz = raw_key(P[0]) != (K)0;  // false too where there is no candidate
         prp = nz ? rp : T(1);
