@@ -507,7 +507,7 @@ extern "C" int32_t rlu_factor_batched(rlu_batch* b, void* stream) {
                                 b->count_y, b->wide_y, s, b->have_fork ? &b->lu_fork : nullptr));
   RLU_TRY(build_ly_batched(reinterpret_cast<const BuildJob*>(ws + t.build), c, b->max_m,
                            b->max_k, s));
-  if (t.small_k)  // the Gram is k x k with k <= 64: one CTA per problem
+  if (t.small_k)  // the Gram is k x k with k <= 64: up to two CTAs per problem
     RLU_TRY(gram_small_batched(reinterpret_cast<const GemmArgs*>(ws + t.gemm_g), c, s));
   else
     RLU_TRY((gemm_simt_batched<float, double>(reinterpret_cast<const GemmArgs*>(ws + t.gemm_g),

@@ -41,9 +41,9 @@ int32_t launch_lu_reg(int32_t dtype, bool crout, const LuArgs& a, cudaStream_t s
 // Batched FP32 LUs of single-panel problems (C <= 76, R <= 16 x rows_per_cta), one cluster
 // each; the device table is grouped (entries first[g] .. first[g] + count[g] - 1; first and
 // count are host arrays of kLuGroups entries): g = 1..16 is the cluster size ceil(R /
-// rows_per_cta) with rows_per_cta-thread CTAs, g = 17 one 128-thread CTA (R <= 128), g = 18
-// one 256-thread CTA (R <= 256). Each entry carries its rpc (rows per CTA), p0 = 0, pw = C
-// and its own position state (posg, psg).
+// rows_per_cta), g = 17 one CTA for R <= 128, g = 18 one CTA for R <= 256; every CTA has 128
+// control and 128 update threads. Each entry carries its rpc (rows per CTA), p0 = 0, pw = C and
+// its own position state (posg, psg).
 static constexpr int kLuGroups = 19;
 // Helper streams for the groups: with fork != nullptr every non-empty group is launched on
 // its own helper stream (fork / join events around them on s), so that the groups' CTAs
