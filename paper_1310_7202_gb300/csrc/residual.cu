@@ -14,12 +14,15 @@
 // the exact rounding error of every addition carried down (Knuth's two-sum), so that nothing
 // above 2^-70 or so of the terms is dropped, where FP64 rounds every addition at 2^-53. It
 // holds while no term leaves the FP32 range; k_range looks for the largest magnitudes of A, L
-// and U first, and outside [2^-20, 2^40] (also for Inf, NaN and all-zero operands) the passes
-// take their FP64 form.
+// and U first. Where one is outside [2^-20, 2^40] (also for Inf, NaN and all-zero operands), or
+// where by them A times y = (PAQ - LU) x, ||x|| = 1, could pass 2^126 in a sum over a chunk of
+// rows (y is not known beforehand), the passes take their FP64 form.
 #include "common.cuh"
 #include "residual.cuh"
 
 namespace rlu {
+
+static constexpr int RS_RB = 64;  // row blocks of the transposed product
 
 template <typename T> __device__ __forceinline__ double to_d(T v) { return (double)v; }
 template <> __device__ __forceinline__ double to_d<__nv_bfloat16>(__nv_bfloat16 v) {
@@ -80,9 +83,12 @@ __device__ __forceinline__ bool in_range(const uint32_t* mx) {
 }
 
 // Largest |entry| of A, L (m x k column-major) and U (k x n row-major) as float bits (a NaN
-// counts as larger than Inf) in mx[0..2], zero on entry.
+// counts as larger than Inf) in mx[0..2]; mx[0] = 0, out of range, where the three together allow
+// too large a product (lu_exp and top_exp: range_limits). mx[3] counts blocks; all four are zero
+// on entry.
 template <typename TA, typename TLU>
-__global__ void __launch_bounds__(256) k_range(ResidualArgs a, uint32_t* __restrict__ mx) {
+__global__ void __launch_bounds__(256) k_range(ResidualArgs a, int lu_exp, int top_exp,
+                                               uint32_t* __restrict__ mx) {
   uint32_t big[3] = {0, 0, 0};
   auto scan = [&](auto* p, int64_t rows, int64_t cols, int64_t ld, uint32_t& b) {
     for (int64_t r = blockIdx.x; r < rows; r += gridDim.x)
@@ -98,6 +104,26 @@ __global__ void __launch_bounds__(256) k_range(ResidualArgs a, uint32_t* __restr
     const uint32_t w = __reduce_max_sync(0xffffffffu, big[i]);
     if ((threadIdx.x & 31) == 0 && w) atomicMax(mx + i, w);
   }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(mx + 3, 1u) == gridDim.x - 1) {  // the last block
+    __threadfence();
+    int e[3];
+    for (int i = 0; i < 3; ++i) e[i] = (int)(__ldcg(mx + i) >> 23);
+    if (e[0] + max(e[0], e[1] + e[2] + lu_exp) > top_exp) mx[0] = 0;
+  }
+}
+struct RangeLimits { int lu_exp, top_exp; };
+// |(PAQ - LU) x| <= sqrt(n) (max|A| + k max|L| max|U|), and its products with A over a chunk of
+// rows stay below 2^126; a maximum is below 2^(e - 126), e its exponent field.
+static RangeLimits range_limits(const ResidualArgs& a) {
+  auto log2_up = [](int64_t v) {  // smallest e with v <= 2^e
+    int e = 0;
+    while (((int64_t)1 << e) < v) ++e;
+    return e;
+  };
+  return {log2_up(a.k) - 126,
+          126 + 2 * 126 - 1 - (log2_up(a.n) + 1) / 2 - log2_up(ceil_div(a.m, RS_RB))};
 }
 
 static constexpr int RS_BM = 64, RS_BN = 64, RS_BK = 16;
@@ -514,7 +540,6 @@ __global__ void k_sqrt_into(const double* __restrict__ in, double* __restrict__ 
   out[0] = sqrt(in[0]);
 }
 
-static constexpr int RS_RB = 64;  // row blocks of the transposed product
 
 size_t residual_workspace_bytes(int64_t m, int64_t n, int k) {
   const int64_t tiles = ceil_div(m, RS_BM) * ceil_div(n, RS_BN);
@@ -541,8 +566,10 @@ static int32_t residual_t(const ResidualArgs& a, double* err_fro, double* err_sp
   float* xs = reinterpret_cast<float*>(zpart);
   if (ty > 65535) return RLU_EUNSUPPORTED;
   if (has_f32<TA, TLU>()) {
-    RLU_CUDA_TRY(cudaMemsetAsync(mx, 0, 3 * sizeof(uint32_t), s));
-    k_range<TA, TLU><<<(unsigned)std::min<int64_t>(std::max<int64_t>(a.m, a.k), 16 * sm_count()), 256, 0, s>>>(a, mx);
+    RLU_CUDA_TRY(cudaMemsetAsync(mx, 0, 4 * sizeof(uint32_t), s));
+    const RangeLimits lim = range_limits(a);
+    k_range<TA, TLU><<<(unsigned)std::min<int64_t>(std::max<int64_t>(a.m, a.k), 16 * sm_count()), 256, 0, s>>>(
+        a, lim.lu_exp, lim.top_exp, mx);
     RLU_TRY(last_launch_status());
   }
   k_residual_fro<TA, TLU><<<dim3((unsigned)tx, (unsigned)ty), 256, 0, s>>>(a, partial, mx);

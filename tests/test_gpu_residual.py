@@ -52,3 +52,21 @@ def test_zero():
         t.zero_()
     fro, spec = rlu.reconstruct_error(*args, power_iters=3)
     assert float(fro) == 0.0 and float(spec) == 0.0
+
+
+# All of one sign, so that y = (PAQ - LU) x adds up: |y| reaches k 2^(2e) sqrt(n), and A y and its
+# sums over a chunk of rows leave the FP32 range although A, L and U are far inside it. Tolerances
+# as in test_norms; the residual is of the size of L U, so no cancellation loosens them.
+@pytest.mark.parametrize("m,n,k,e", [(200, 190, 20, 40), (2000, 1500, 100, 38), (2000, 1500, 100, 36),
+                                     (300, 257, 40, 28), (257, 300, 3, 39)])
+def test_large_factors_of_one_sign(m, n, k, e):
+    rng = np.random.default_rng(m + e)
+    L, U, A = (np.ldexp(rng.uniform(0.5, 1.0, s), e).astype(np.float32) for s in ((m, k), (k, n), (m, n)))
+    P, Q = rng.permutation(m).astype(np.int32), rng.permutation(n).astype(np.int32)
+    Lt = torch.from_numpy(np.ascontiguousarray(L.T)).cuda().t()
+    fro, spec = rlu.reconstruct_error(*(torch.from_numpy(x).cuda() for x in (A, P, Q)), Lt,
+                                      torch.from_numpy(U).cuda(), power_iters=60)
+    R = A.astype(np.float64)[P][:, Q] - L.astype(np.float64) @ U.astype(np.float64)
+    want, top = np.linalg.norm(R), np.linalg.norm(R, 2)
+    assert abs(float(fro) - want) <= 1e-12 * want
+    assert top * 0.97 <= float(spec) <= top * (1 + 1e-12)
