@@ -12,7 +12,7 @@
 //   and B = Q^T A, so that Q B = Q Q^T A is the rank-k approximation whose error
 //   ||Q Q^T A - A|| Section 5 compares with the randomized LU's.
 //
-// The Jacobi eigensolver (parallel two-sided Jacobi; k_jacobi_smem for l <= 112, k_jacobi_sym
+// The Jacobi eigensolver (parallel two-sided Jacobi; k_jacobi_smem for l <= 80, k_jacobi_sym
 // above): the l x l matrix (l rounded up to an
 // even l2; a padding index stays decoupled) is swept by the round-robin (circle) schedule:
 // each round pairs every index with one other, and the l2 / 2 rotations of a round commute,
@@ -191,7 +191,12 @@ __global__ void __launch_bounds__(JAC_T) k_jacobi_sym(JacArgs a) {
 //
 // With d = m_qq - m_pp, b = 2 m_pq and h = sqrt(d^2 + b^2), the smaller rotation that zeroes
 // m_pq has cos 2phi = |d| / h: c = sqrt((1 + |d| / h) / 2), s = sign(d) b / (2 h c).
-static constexpr int JAC_SMEM_MAX = 112;
+//
+// One SM does all the FP64 work here, which k_jacobi_sym spreads over several at the price of
+// grid barriers, so the two cross before shared memory ends (l2 = 112): rlu_rsvd at 3000 x 3000,
+// this form against that one, takes 2.9 / 4.8 ms at l = 43, 5.7 / 7.6 at 64, 9.0 / 10.4 at 72,
+// 10.7 / 10.7 at 80, 11.7 / 11.2 at 84, 18.2 / 13.0 at 104.
+static constexpr int JAC_SMEM_MAX = 80;
 static constexpr int JAC_ST = 512;
 
 static size_t jac_smem_bytes(int l2) {
@@ -488,15 +493,14 @@ extern "C" int32_t rlu_rsvd(const void* A, int32_t dtype, int64_t m, int64_t n, 
   ja.status = status;
   if (l2 <= JAC_SMEM_MAX) {
     const size_t smem = jac_smem_bytes(l2);
-    RLU_CUDA_TRY(cudaFuncSetAttribute(k_jacobi_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+    RLU_TRY(allow_smem(k_jacobi_smem));
     k_jacobi_smem<<<1, JAC_ST, smem, s>>>(ja);
     RLU_TRY(last_launch_status());
   } else {
     const int P = l2 / 2;
     const size_t smem = (size_t)P * (sizeof(double2) + sizeof(int2));
     const void* fn = reinterpret_cast<const void*>(&k_jacobi_sym);
-    RLU_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RLU_TRY(allow_smem(fn));
     int per_sm = 0;
     RLU_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, JAC_T, smem));
     if (per_sm < 1) return RLU_EUNSUPPORTED;

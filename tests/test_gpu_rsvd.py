@@ -104,3 +104,56 @@ def test_rsvd_rejects_bad_arguments():
     A = torch.zeros((64, 48), dtype=torch.float32, device="cuda")
     with pytest.raises(rlu.RluError):
         rlu.rsvd(A, 4, 6, 1)                                     # FP64 only
+
+
+def test_rsvd_time_does_not_fall_with_l():
+    """A problem with fewer vectors is no slower than one with more. The eigensolver's sweeps
+    depend on the data (here one of about nine more or less) and its rounds are l - 1, so the
+    smaller l gets 20% of slack, less where it is far below the larger."""
+    A = torch.randn(600, 500, dtype=torch.float64, device="cuda",
+                    generator=torch.Generator("cuda").manual_seed(3))
+    ls = list(range(64, 137, 8))
+    t = {}
+    for l in ls:
+        rlu.rsvd(A, l, l, 5)
+        best = float("inf")
+        for _ in range(4):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            e0.record()
+            rlu.rsvd(A, l, l, 5)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        t[l] = best
+    slow = [(a, b) for a in ls for b in ls if a < b and t[a] > 1.2 * t[b]]
+    assert not slow, t
+
+
+@pytest.mark.parametrize("l", [1, 2, 3, 63, 64, 65, 66, 79, 80, 81, 82, 95, 96, 97, 111, 112, 113])
+def test_rsvd_around_the_eigensolvers_sizes(l):
+    """One index, one pair, and the sizes around multiples of 16 where the number of CTAs of the
+    eigensolver or its form may change; tolerances of test_rsvd_matches_the_oracle."""
+    m, n = 300, 260
+    A = synth.prescribed_matrix(m, n, synth.spectrum("paper_slow", n), 13, 14)
+    k = max(1, l - 3)
+    _, g, _ = _run(A, k, l, 9)
+    sy = O.randomized_orth(A, k, l, seed=9)["sigma_y"]
+    assert g["info"].tolist()[0] == 0
+    assert np.abs(g["sigma"] - sy).max() <= 1e-9 * sy[0]
+    assert np.abs(g["Q"].T @ g["Q"] - np.eye(k)).max() <= 1e-10
+
+
+@pytest.mark.parametrize("e", [-250, 250])
+@pytest.mark.parametrize("l", [30, 121])
+def test_rsvd_far_from_one(l, e):
+    """A scaled by 2^e, so that products of two entries of the Gram matrix leave the FP64 range:
+    the factors scale along (a power of two rounds nothing)."""
+    m, n = 300, 260
+    A = synth.prescribed_matrix(m, n, synth.spectrum("paper_slow", n), 13, 14)
+    _, one, _ = _run(A, l, l, 9)
+    _, g, _ = _run(np.ldexp(A, e), l, l, 9)
+    assert g["info"].tolist()[0] == 0
+    want = np.ldexp(one["sigma"], e)
+    assert np.abs(g["sigma"] - want).max() <= 1e-9 * want[0]
+    assert np.abs(g["Q"].T @ g["Q"] - np.eye(l)).max() <= 1e-10
