@@ -533,7 +533,7 @@ static int32_t clu_coop(bool crout, float2* Y, int64_t ldy, int rows, int cols, 
   const size_t smem = clu_smem_bytes(rloc, cols);
   const void* fn = crout ? reinterpret_cast<const void*>(&k_clu_coop<true>)
                          : reinterpret_cast<const void*>(&k_clu_coop<false>);
-  RLU_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  RLU_TRY(allow_smem(fn));
   int per_sm = 0;
   RLU_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, CLU_T, smem));
   if (per_sm * sm_count() < G) return RLU_EUNSUPPORTED;
@@ -696,8 +696,7 @@ template <int NS>
 static int32_t wsolve_launch(const double* V, int64_t ldv, int k, int l, const float2* Y,
                              int64_t ldy, float* Wst, int64_t ldw, cudaStream_t s) {
   const size_t smem = 32 * 32 * NS * sizeof(float2);
-  RLU_CUDA_TRY(cudaFuncSetAttribute(k_frlu_wsolve<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem));
+  RLU_TRY(allow_smem(k_frlu_wsolve<NS>));
   k_frlu_wsolve<NS><<<(unsigned)ceil_div(k, WS_ROWS), WS_T, smem, s>>>(V, ldv, k, l, Y, ldy, Wst,
                                                                        ldw);
   return last_launch_status();
@@ -967,7 +966,7 @@ static int32_t srft_apply(const float* A, int64_t m, int64_t n, int64_t lda, con
   const float scale = (float)(1.0 / std::sqrt((double)n));
   // the narrowest register array that holds n values over FFT_T threads
   auto go = [&](auto kern) -> int32_t {
-    RLU_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
+    RLU_TRY(allow_smem(kern));
     kern<<<(unsigned)m, FFT_T, fsmem, s>>>(A, lda, (int)n, d, sel, l, scale, f, Y, ldy, status);
     return last_launch_status();
   };

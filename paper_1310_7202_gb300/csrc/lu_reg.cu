@@ -1141,8 +1141,7 @@ static int32_t launch_trail(T* X, int64_t ldx, int R, int c_begin, int c_end, in
   int nch = 1;
   while (nch < 4 && (int64_t)rows * ceil_div(chunks, nch + 1) >= 2 * sm_count()) ++nch;
   const size_t smem = sizeof(T) * (size_t)w * (TR_R + 2 * LR_CH);
-  RLU_CUDA_TRY(cudaFuncSetAttribute(k_lu_trail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem));
+  RLU_TRY(allow_smem(k_lu_trail<T>));
   const bool vec = ((uintptr_t)X % 16 == 0) && (ldx * (int64_t)sizeof(T)) % 16 == 0;
   const dim3 grid((unsigned)rows, (unsigned)ceil_div(chunks, nch));
   k_lu_trail<T><<<grid, TR_T, smem, s>>>(X, ldx, R, c_begin, c_end, p0, w, posg, u12, ldu, nch,
@@ -1193,7 +1192,7 @@ static int32_t try_launch(const LuArgs& in, cudaStream_t s, bool* launched) {
   const size_t bytes = lr_smem_bytes<T, RT, NC>(pw, in.C > wo ? wo : in.C > pw ? pw : 0);
   if (bytes > (size_t)optin) return RLU_OK;
   auto kern = k_lu_reg<T, CROUT, RT, NC, SOLO>;
-  RLU_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  RLU_TRY(allow_smem(kern));
   RLU_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
@@ -1302,7 +1301,7 @@ static int32_t lu_batched_group(bool crout, const LuArgs* table_dev, int first, 
                               : k_lu_reg_batched<T, false, RT, NC, true>)
                     : (crout ? k_lu_reg_batched<T, true, RT, NC, false>
                              : k_lu_reg_batched<T, false, RT, NC, false>);
-  RLU_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  RLU_TRY(allow_smem(kern));
   RLU_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];

@@ -289,19 +289,14 @@ __global__ void __launch_bounds__(LU_NT, 1) k_cluster_lu(LuArgs a) {
 // ---------------------------------------------------------------------------------------
 template <typename T, bool CROUT>
 static int32_t launch_lu_t(const LuArgs& in, cudaStream_t s) {
-  static bool attr_done[64] = {false};
   int dev = 0;
   RLU_CUDA_TRY(cudaGetDevice(&dev));
   int smem_optin = 0;
   RLU_CUDA_TRY(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   const size_t budget = (size_t)smem_optin - 2048;  // static shared memory and slack
   auto kern = k_cluster_lu<T, CROUT>;
-  if (dev < 64 && !attr_done[dev]) {
-    RLU_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)budget));
-    RLU_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    attr_done[dev] = true;
-  }
+  RLU_TRY(allow_smem(kern));
+  RLU_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   const int R = in.R, C = in.C;
   auto launchable = [&](int cand, size_t bytes) -> bool {
     if (cand <= 8) return true;  // portable cluster sizes

@@ -13,6 +13,7 @@
 #include <atomic>
 #include <map>
 #include <mutex>
+#include <set>
 #include <utility>
 
 #include "common.cuh"
@@ -54,6 +55,22 @@ int sm_count() {
   if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 1;
   if (dev >= 0 && dev < 64) cached[dev] = n;
   return n;
+}
+
+int32_t allow_smem_of(const void* kernel) {
+  static std::mutex mu;
+  static std::set<std::pair<int, const void*>> done;
+  int dev = 0, optin = 0;
+  RLU_CUDA_TRY(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lock(mu);
+  if (done.count({dev, kernel})) return RLU_OK;
+  cudaFuncAttributes at{};
+  RLU_CUDA_TRY(cudaFuncGetAttributes(&at, kernel));
+  RLU_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  RLU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    optin - (int)at.sharedSizeBytes));
+  done.insert({dev, kernel});
+  return RLU_OK;
 }
 
 int32_t side_stream(cudaStream_t main, SideStream** out) {

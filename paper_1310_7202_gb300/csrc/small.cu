@@ -583,7 +583,7 @@ static int32_t ldl_cluster_f64(double* M, int k, double* dinv, int32_t* status, 
   while (nc < 16 && bytes_for(nc) + 1024 > (size_t)optin) ++nc;
   const size_t bytes = bytes_for(nc);
   if (bytes + 1024 > (size_t)optin) return RLU_EUNSUPPORTED;
-  RLU_CUDA_TRY(cudaFuncSetAttribute(k_chol_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  RLU_TRY(allow_smem(k_chol_cluster));
   RLU_CUDA_TRY(cudaFuncSetAttribute(k_chol_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
@@ -771,7 +771,7 @@ static int32_t ldl32_cluster(const double* M, int k, const LdlOut<float>& o, int
   int optin = 0;
   RLU_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   if (bytes + 1024 > (size_t)optin) return RLU_EUNSUPPORTED;
-  RLU_CUDA_TRY(cudaFuncSetAttribute(k_ldl32c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  RLU_TRY(allow_smem(k_ldl32c));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -792,7 +792,7 @@ template <typename T>
 int32_t ldl_factor(double* M, int k, const LdlOut<T>& o, int32_t* status, cudaStream_t s) {
   if (sizeof(T) == sizeof(float) && k <= L32_MAXB * LB) {
     const size_t bytes = ldl32_smem_bytes(k);
-    RLU_CUDA_TRY(cudaFuncSetAttribute(k_ldl32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    RLU_TRY(allow_smem(k_ldl32));
     k_ldl32<<<1, L32_NT, bytes, s>>>(M, k, reinterpret_cast<const LdlOut<float>&>(o), status);
     return last_launch_status();
   }
@@ -1261,8 +1261,7 @@ template <typename T, int TC, int TR = 8>
 static int32_t trsm_rl_launch(const LdlOut<T>& o, const T* C, int64_t ldc, int64_t n, T* B,
                               int64_t ldb, cudaStream_t s) {
   const size_t bytes = trsm_rl_smem_bytes<T>(o.kp, TC);
-  RLU_CUDA_TRY(cudaFuncSetAttribute(k_trsm_rl<T, TC, TR>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  RLU_TRY(allow_smem(k_trsm_rl<T, TC, TR>));
   k_trsm_rl<T, TC, TR><<<(unsigned)ceil_div(n, TC), RL_NT<T>, bytes, s>>>(o, C, ldc, n, B, ldb);
   return last_launch_status();
 }
@@ -1275,8 +1274,7 @@ static size_t trsm_smem_bytes(int kp, int tc) {
 template <typename T, int TC>
 static int32_t trsm_launch(const LdlOut<T>& o, const T* C, int64_t ldc, int64_t n, T* B,
                            int64_t ldb, size_t bytes, cudaStream_t s) {
-  RLU_CUDA_TRY(cudaFuncSetAttribute(k_trsm_ldl<T, TC>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  RLU_TRY(allow_smem(k_trsm_ldl<T, TC>));
   k_trsm_ldl<T, TC><<<(unsigned)ceil_div(n, TC), TB / 2 * TC / 4, bytes, s>>>(o, C, ldc, n, B,
                                                                               ldb);
   return last_launch_status();
@@ -1453,8 +1451,7 @@ int32_t build_ly_batched(const BuildJob* jobs_dev, int count, int64_t max_m, int
   const bool four = max_m <= BG_LONG;
   const auto kernel = four ? k_build_ly_batched<4> : k_build_ly_batched<1>;
   const size_t smem = (size_t)max_m * sizeof(float) * (four ? 4 : 1);
-  RLU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem));
+  RLU_TRY(allow_smem(kernel));
   kernel<<<dim3((unsigned)count, 8), 256, smem, s>>>(jobs_dev);
   return last_launch_status();
 }
@@ -1550,12 +1547,10 @@ int32_t ldl32_batched(const Ldl32Job* jobs_dev, int count, int max_k, cudaStream
   if (max_k > L32_MAXB * LB) return RLU_EUNSUPPORTED;
   const size_t bytes = ldl32_smem_bytes(max_k);
   if (max_k <= 4 * LB) {
-    RLU_CUDA_TRY(cudaFuncSetAttribute(k_ldl32_batched<128>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    RLU_TRY(allow_smem(k_ldl32_batched<128>));
     k_ldl32_batched<128><<<(unsigned)count, 128, bytes, s>>>(jobs_dev);
   } else {
-    RLU_CUDA_TRY(cudaFuncSetAttribute(k_ldl32_batched<L32_NT>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    RLU_TRY(allow_smem(k_ldl32_batched<L32_NT>));
     k_ldl32_batched<L32_NT><<<(unsigned)count, L32_NT, bytes, s>>>(jobs_dev);
   }
   return last_launch_status();
@@ -1731,8 +1726,7 @@ int32_t trsm_batched(const TrsmJob* jobs_dev, const int2* tiles_dev, int ntiles,
   int optin = 0;
   RLU_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   if (bytes > (size_t)optin) return RLU_EUNSUPPORTED;
-  RLU_CUDA_TRY(cudaFuncSetAttribute(k_trsm_batched, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)bytes));
+  RLU_TRY(allow_smem(k_trsm_batched));
   k_trsm_batched<<<(unsigned)ntiles, TB / 2 * 64 / 4, bytes, s>>>(jobs_dev, tiles_dev);
   return last_launch_status();
 }
@@ -1777,8 +1771,7 @@ int32_t gather_batched(const GatherJob* jobs_dev, int count, int max_k, int64_t 
   const bool four = max_n <= BG_LONG;
   const auto kernel = four ? k_gather_batched<4> : k_gather_batched<1>;
   const size_t smem = (size_t)max_n * sizeof(float) * (four ? 4 : 1);
-  RLU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem));
+  RLU_TRY(allow_smem(kernel));
   kernel<<<dim3((unsigned)count, 8), 256, smem, s>>>(jobs_dev);
   return last_launch_status();
 }

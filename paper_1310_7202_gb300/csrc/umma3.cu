@@ -939,7 +939,7 @@ static int32_t launch_u3(const Umma3Op& op, cudaStream_t s) {
     a.split_stride = (size_t)op.M * op.N;
   }
   auto kern = k_umma3<MODE>;
-  RLU_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  RLU_TRY(allow_smem(kern));
   // x: (row tile, N tile) with the N tile fastest
   dim3 grid((unsigned)(ceil_div(op.M, U3_BM) * ntiles), (unsigned)splits);
   kern<<<grid, U3_THREADS, smem, s>>>(m0, m1, n0, n1, a);
@@ -1022,7 +1022,7 @@ int32_t umma3_batched(int mode, const U3Job* jobs_dev, const int2* tiles_dev, in
   }
   // persistent: as many CTAs as stay resident (one or two per SM), each walking the list
   auto go = [&](auto kern) -> int32_t {
-    RLU_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RLU_TRY(allow_smem(kern));
     int per_sm = 0;
     RLU_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, U3_THREADS, smem));
     if (per_sm < 1) return RLU_EUNSUPPORTED;

@@ -449,7 +449,7 @@ static int32_t launch_ub(const UmmaBf16Op& op, cudaStream_t s) {
     a.split_stride = (size_t)op.M * op.N;
   }
   auto kern = k_ummab<MODE>;
-  RLU_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  RLU_TRY(allow_smem(kern));
   const int rows_per_cta = MODE == UB_MODE_Y ? 2 * UB_BM : UB_BM;
   dim3 grid((unsigned)(ceil_div(op.M, rows_per_cta) * ntiles), (unsigned)splits);
   kern<<<grid, UB_THREADS, smem, s>>>(mA, b0, b1, b2, a);

@@ -515,8 +515,7 @@ int32_t umma_fp8_y(const Fp8Op& op, cudaStream_t s) {
     a.out_colmajor = false;
     a.split_stride = (size_t)op.M * op.N;
   }
-  RLU_CUDA_TRY(cudaFuncSetAttribute(k_umma_fp8, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem));
+  RLU_TRY(allow_smem(k_umma_fp8));
   dim3 grid((unsigned)(ceil_div(op.M, 2 * F8_BM) * ntiles), (unsigned)splits);
   k_umma_fp8<<<grid, F8_THREADS, smem, s>>>(mA, mG, mGl, a);
   RLU_TRY(last_launch_status());
