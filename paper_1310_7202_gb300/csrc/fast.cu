@@ -702,14 +702,16 @@ static int32_t wsolve_launch(const double* V, int64_t ldv, int k, int l, const f
   return last_launch_status();
 }
 
-// A(J,:) (l x n, row-major, ld ldaj): row i is row perm[i] of A.
-__global__ void k_frlu_gather_aj(const float* __restrict__ A, int64_t lda, int n,
+// A(J,:) (l x n, row-major, ld ldaj): row i is row perm[i] of A (m x n); zeros where perm[i] is
+// outside [0, m), an entry that an LU that gave up waiting has left unset.
+__global__ void k_frlu_gather_aj(const float* __restrict__ A, int64_t lda, int m, int n,
                                  const int32_t* __restrict__ perm, float* __restrict__ AJ,
                                  int64_t ldaj) {
   const int i = blockIdx.y;
   const int64_t src = perm[i];
+  const bool in = src >= 0 && src < m;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x)
-    AJ[(int64_t)i * ldaj + c] = A[src * lda + c];
+    AJ[(int64_t)i * ldaj + c] = in ? A[src * lda + c] : 0.f;
 }
 
 // B^T (n x k complex, row-major, ld ldt) from the planes Bst = [Re B; Im B] (2k x n, ld ldb).
@@ -791,7 +793,8 @@ __global__ void k_c_rm_to_cm(const float2* __restrict__ Yr, int64_t ldr, int R, 
 }
 
 // The register LU's swap-free result back to the positional row-major layout of the rest of
-// the pipeline: row p of Yr = row perm[p] of X (column-major, ld ldc).
+// the pipeline: row p of Yr = row perm[p] of X (column-major, ld ldc), zeros where perm[p] is
+// outside [0, R).
 __global__ void k_c_cm_to_rm_perm(const float2* __restrict__ X, int64_t ldc, int R, int C,
                                   const int32_t* __restrict__ perm, float2* __restrict__ Yr,
                                   int64_t ldr) {
@@ -802,7 +805,9 @@ __global__ void k_c_cm_to_rm_perm(const float2* __restrict__ X, int64_t ldc, int
   __syncthreads();
   for (int j = threadIdx.y; j < 32; j += blockDim.y) {  // column c0 + j, rows src[x]
     const int c = c0 + j, p = p0 + threadIdx.x;
-    if (p < R && c < C) t[threadIdx.x][j] = X[(int64_t)c * ldc + src[threadIdx.x]];
+    const int r = src[threadIdx.x];
+    if (p < R && c < C)
+      t[threadIdx.x][j] = r >= 0 && r < R ? X[(int64_t)c * ldc + r] : make_float2(0.f, 0.f);
   }
   __syncthreads();
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
@@ -1059,7 +1064,7 @@ static int32_t fast_factor(const FastPlan& p, const float* A, int64_t m, int64_t
       RLU_TRY(st);
     }
     k_frlu_gather_aj<<<dim3((unsigned)std::min<int64_t>(ceil_div(n, 256), 64), (unsigned)l), 256, 0, s>>>(
-        A, lda, (int)n, P, AJ, p.ldn);
+        A, lda, (int)m, (int)n, P, AJ, p.ldn);
     RLU_TRY(last_launch_status());
     if (p.tc) {  // C^T = A(J,:)^T W^T: A(J,:) as the raw n-contiguous operand, W's TF32 parts
       float* Wh = reinterpret_cast<float*>(ws + p.off_Wh);

@@ -1308,6 +1308,7 @@ template int32_t trsm_ldl<double>(const LdlOut<double>&, const double*, int64_t,
 // rows a thread (they share Q[j], and their gathers are in flight together). Grid rows past
 // U's write L_b (k x k): L_b[i][j] = B[i][Q[j]] for i > j, 1 on the diagonal, 0 above, as it is
 // (Lb, column-major, ld k) and / or as its TF32 parts (Lbh, Lbl, ld ldh). B is row-major k x n.
+// An entry of Q outside [0, n), which an LU that gave up waiting leaves, reads zeros.
 template <typename T>
 __global__ void __launch_bounds__(256) k_gather_lb_u(const T* __restrict__ B, int64_t ldb,
                                                      const int32_t* __restrict__ Q, int k,
@@ -1320,10 +1321,11 @@ __global__ void __launch_bounds__(256) k_gather_lb_u(const T* __restrict__ B, in
     const int i0 = 4 * (int)blockIdx.y;
     for (int64_t j = x; j < n; j += gridDim.x * 256ll) {
       const int64_t q = Q[j];
+      const bool in = q >= 0 && q < n;
       T v[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        v[u] = i0 + u < k && j >= i0 + u ? B[(int64_t)(i0 + u) * ldb + q] : T(0);
+        v[u] = in && i0 + u < k && j >= i0 + u ? B[(int64_t)(i0 + u) * ldb + q] : T(0);
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (i0 + u < k) U[(int64_t)(i0 + u) * ldu + j] = v[u];
@@ -1334,7 +1336,8 @@ __global__ void __launch_bounds__(256) k_gather_lb_u(const T* __restrict__ B, in
   for (int64_t e = ((int64_t)(blockIdx.y - ub) * gridDim.x) * 256 + x; e < (int64_t)k * k;
        e += threads) {
     const int j = (int)(e / k), i = (int)(e % k);
-    const T v = i > j ? B[(int64_t)i * ldb + Q[j]] : (i == j ? T(1) : T(0));
+    const int64_t q = Q[j];
+    const T v = i > j && q >= 0 && q < n ? B[(int64_t)i * ldb + q] : (i == j ? T(1) : T(0));
     if (Lb) Lb[e] = v;
     if (Lbh) tf32_split(v, Lbh, Lbl, (int64_t)j * ldh + i);
   }
