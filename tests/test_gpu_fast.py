@@ -143,3 +143,20 @@ def test_fast_factor_benchmark_size_properties():
     assert fro_fast <= 10 * fro_rlu + 1e-4 * sigma[0], (fro_fast, fro_rlu)
     bound = (1 + math.sqrt(1 + 4 * k * (n - k))) * math.sqrt(1 + 7 * n / l) * sigma[k]
     assert spec_fast <= bound
+
+
+@pytest.mark.parametrize("m,n,k,l", [(4097, 240, 20, 40), (4100, 240, 40, 80), (8193, 200, 16, 24),
+                                     (16388, 160, 20, 40)])
+def test_fast_factor_tall(m, n, k, l):
+    """More rows than two, four and eight rows a thread of the complex LU hold (4096, 8192 and
+    16384), with panels of 36, 18 and 8 columns; the tolerances of test_fast_factor_against_oracle."""
+    sigma = synth.spectrum("exp_k", n, k)
+    A = synth.prescribed_matrix(m, n, sigma, m, n, dtype=np.float32)
+    g, theta, s = _factor(A, k, l, seed=k)
+    o = F.frlu_factor(A.astype(np.float64), k, l, theta, s)
+    fro_o, _ = F.creconstruct_error(A, o["P"], o["Q"], o["L"], o["U"])
+    fro_g, _ = F.creconstruct_error(A, g["P"], g["Q"], g["L"], g["U"])
+    assert fro_g <= 1.1 * fro_o + 1e-4 * sigma[0], (fro_g, fro_o)
+    assert sorted(g["P"].tolist()) == list(range(m)) and sorted(g["Q"].tolist()) == list(range(n))
+    assert leading_agreement(g["P"], o["P"], l) >= 5
+    assert g["info"].tolist()[:3] == [0, -1, -1]

@@ -36,3 +36,13 @@ def test_f32_edges(m, n, k, l):
     fro, _ = O.reconstruct_error(A64, g["P"], g["Q"], g["L"], g["U"], spectral=False)
     fro_or, _ = O.reconstruct_error(A64, o["P"], o["Q"], o["L"], o["U"], spectral=False)
     assert fro <= 1.1 * fro_or + 1e-4 * O.spectral_norm(A64)
+
+
+@pytest.mark.parametrize("m,n,k,l", [(16385, 60, 20, 26), (40, 16390, 20, 30)])
+def test_f64_tallest_form(m, n, k, l):
+    """Eight rows a thread with panels of 8 columns, for the LU of Y and for that of B^T."""
+    A = synth.lowrank_plus_noise(m, n, min(m, n), 1e-3, seed=m + l)
+    g, o = run_gpu(A, k, l, 5, "f64"), oracle_for(A, k, l, 5, "f64")
+    assert g["info"].tolist() == [0, -1, -1, 0]
+    assert np.array_equal(g["P"], o["P"]) and np.array_equal(g["Q"], o["Q"])
+    assert rel_max(g["L"], o["L"]) <= 1e-10 and rel_max(g["U"], o["U"]) <= 1e-10
