@@ -244,7 +244,7 @@ __device__ __forceinline__ double residual_tile_f64(const ResidualArgs& a,
   return sq;
 }
 
-template <typename TA, typename TLU>
+template <typename TA, typename TLU, bool F32>
 __global__ void __launch_bounds__(256) k_residual_fro(ResidualArgs a, double* __restrict__ partial,
                                                       const uint32_t* __restrict__ mx) {
   __shared__ double tiles[2][RS_BK][RS_BM + 1];
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(256) k_residual_fro(ResidualArgs a, double* __
   const int tid = threadIdx.x;
   double sq;
   bool done = false;
-  if constexpr (has_f32<TA, TLU>()) {
+  if constexpr (F32) {
     if (in_range(mx)) {
       sq = residual_tile_f32<TA>(a, reinterpret_cast<float(*)[RS_BM + 1]>(&tiles[0][0][0]),
                                  reinterpret_cast<float(*)[RS_BN + 1]>(&tiles[1][0][0]));
@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(256) k_l_u(ResidualArgs a, const double* __res
 }
 
 // y[i] = sum_c A[P[i]][c] xq[c] - y[i]  (a warp per RB rows; xs: x's float parts)
-template <typename TA, typename TLU, int RB>
+template <typename TA, typename TLU, int RB, bool F32>
 __global__ void __launch_bounds__(256) k_rows(ResidualArgs a, const double* __restrict__ xq,
                                               const float* __restrict__ xs,
                                               double* __restrict__ y,
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(256) k_rows(ResidualArgs a, const double* __re
 #pragma unroll
     for (int b = 0; b < RB; ++b) row[b] = A + (int64_t)a.P[min(i0 + b, a.m - 1)] * a.lda;
     bool done = false;
-    if constexpr (has_f32<TA, TLU>()) {
+    if constexpr (F32) {
       if (in_range(mx)) {
         Acc3 acc[RB];
 #pragma unroll
@@ -462,7 +462,7 @@ __global__ void k_lt_y(const TLU* __restrict__ L, int64_t ldl, const double* __r
 
 // zpart[rb][c] = sum over rows i of chunk rb of A[P[i]][c] y[i]  (thread per column; the rows'
 // offsets and y, with its float parts, staged in shared memory)
-template <typename TA, typename TLU>
+template <typename TA, typename TLU, bool F32>
 __global__ void __launch_bounds__(256) k_cols(ResidualArgs a, const double* __restrict__ y,
                                               int64_t rows_per, double* __restrict__ zpart,
                                               const uint32_t* __restrict__ mx) {
@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(256) k_cols(ResidualArgs a, const double* __re
   const int64_t rb = blockIdx.y;
   const int64_t i0 = rb * rows_per, i1 = min(a.m, i0 + rows_per);
   bool fast = false;
-  if constexpr (has_f32<TA, TLU>()) fast = in_range(mx);
+  if constexpr (F32) fast = in_range(mx);
   Acc3 acc{0.f, 0.f, 0.f};
   double s = 0.0;
   const TA* col = A + (c < a.n ? c : 0);
@@ -548,9 +548,9 @@ size_t residual_workspace_bytes(int64_t m, int64_t n, int k) {
   return (size_t)doubles * sizeof(double);
 }
 
-template <typename TA, typename TLU>
-static int32_t residual_t(const ResidualArgs& a, double* err_fro, double* err_spec, int iters,
-                          double* ws, cudaStream_t s) {
+template <typename TA, typename TLU, bool F32>
+static int32_t residual_run(const ResidualArgs& a, double* err_fro, double* err_spec, int iters,
+                            double* ws, cudaStream_t s) {
   const int64_t tx = ceil_div(a.n, RS_BN), ty = ceil_div(a.m, RS_BM);
   double* partial = ws;
   double* x = partial + round_up(tx * ty, 32);
@@ -565,14 +565,14 @@ static int32_t residual_t(const ResidualArgs& a, double* err_fro, double* err_sp
   // x's float parts, dead before the transposed product writes zpart
   float* xs = reinterpret_cast<float*>(zpart);
   if (ty > 65535) return RLU_EUNSUPPORTED;
-  if (has_f32<TA, TLU>()) {
+  if constexpr (F32) {
     RLU_CUDA_TRY(cudaMemsetAsync(mx, 0, 4 * sizeof(uint32_t), s));
     const RangeLimits lim = range_limits(a);
     k_range<TA, TLU><<<(unsigned)std::min<int64_t>(std::max<int64_t>(a.m, a.k), 16 * sm_count()), 256, 0, s>>>(
         a, lim.lu_exp, lim.top_exp, mx);
     RLU_TRY(last_launch_status());
   }
-  k_residual_fro<TA, TLU><<<dim3((unsigned)tx, (unsigned)ty), 256, 0, s>>>(a, partial, mx);
+  k_residual_fro<TA, TLU, F32><<<dim3((unsigned)tx, (unsigned)ty), 256, 0, s>>>(a, partial, mx);
   RLU_TRY(last_launch_status());
   k_sum_sqrt<<<1, 256, 0, s>>>(partial, tx * ty, err_fro, true);
   RLU_TRY(last_launch_status());
@@ -592,10 +592,10 @@ static int32_t residual_t(const ResidualArgs& a, double* err_fro, double* err_sp
     k_scatter_q<<<gn, threads, 0, s>>>(z, sq, gz, a.Q, a.n, x, xq, xs);
     k_u_x<TLU><<<a.k, 256, 0, s>>>(static_cast<const TLU*>(a.U), a.ldu, x, a.n, u);
     k_l_u<TLU><<<(unsigned)ceil_div(a.m, 64), 256, 0, s>>>(a, u, y);
-    if (rbw == 2) k_rows<TA, TLU, 2><<<gm, threads, 0, s>>>(a, xq, xs, y, mx);
-    else k_rows<TA, TLU, 1><<<gm, threads, 0, s>>>(a, xq, xs, y, mx);
+    if (rbw == 2) k_rows<TA, TLU, 2, F32><<<gm, threads, 0, s>>>(a, xq, xs, y, mx);
+    else k_rows<TA, TLU, 1, F32><<<gm, threads, 0, s>>>(a, xq, xs, y, mx);
     k_lt_y<TLU><<<a.k, 256, 0, s>>>(static_cast<const TLU*>(a.L), a.ldl, y, a.m, v);
-    k_cols<TA, TLU><<<dim3((unsigned)ceil_div(a.n, threads), RS_RB), threads, 0, s>>>(a, y, rows_per, zpart, mx);
+    k_cols<TA, TLU, F32><<<dim3((unsigned)ceil_div(a.n, threads), RS_RB), threads, 0, s>>>(a, y, rows_per, zpart, mx);
     k_finish_z<TLU><<<gz, 512, 0, s>>>(a, zpart, RS_RB, v, z, sq);
     RLU_TRY(last_launch_status(7));
   }
@@ -604,6 +604,19 @@ static int32_t residual_t(const ResidualArgs& a, double* err_fro, double* err_sp
   // ||R^T R x|| with ||x|| = 1 converges to sigma_max^2
   k_sqrt_into<<<1, 1, 0, s>>>(nrm, err_spec);
   return last_launch_status();
+}
+
+// Up to one tile for every SM and one chunk of k, the FP64 form takes less than k_range, its
+// memset and the FP32 form: ||R||_F alone, in a row of calls, 36-38 us against 41 at 300 x 300 to
+// 700 x 700, k = 4 or 16; at k = 64 85 against 62, at 1000 x 1000, k = 16 54 against 51.
+template <typename TA, typename TLU>
+static int32_t residual_t(const ResidualArgs& a, double* err_fro, double* err_spec, int iters,
+                          double* ws, cudaStream_t s) {
+  if constexpr (has_f32<TA, TLU>()) {
+    if (a.k > RS_BK || ceil_div(a.n, RS_BN) * ceil_div(a.m, RS_BM) > sm_count())
+      return residual_run<TA, TLU, true>(a, err_fro, err_spec, iters, ws, s);
+  }
+  return residual_run<TA, TLU, false>(a, err_fro, err_spec, iters, ws, s);
 }
 
 int32_t residual_error(int32_t dtA, int32_t dtLU, const ResidualArgs& a, double* err_fro,

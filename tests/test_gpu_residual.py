@@ -70,3 +70,18 @@ def test_large_factors_of_one_sign(m, n, k, e):
     want, top = np.linalg.norm(R), np.linalg.norm(R, 2)
     assert abs(float(fro) - want) <= 1e-12 * want
     assert top * 0.97 <= float(spec) <= top * (1 + 1e-12)
+
+
+# up to one 64 x 64 tile an SM and 16 columns of L the FP64 form runs, without the scan of the
+# operands' magnitudes; from there on the FP32 form
+@pytest.mark.parametrize("m,n,k,launches", [(300, 257, 16, 2), (300, 257, 17, 3), (640, 576, 16, 2),
+                                            (2000, 1200, 16, 3)])
+def test_small_problems_take_no_scan(m, n, k, launches):
+    args, R = case(m, n, k, torch.float32, 1.0, m + k)
+    before = rlu.launch_count()
+    fro, _ = rlu.reconstruct_error(*args)
+    assert rlu.launch_count() - before == launches
+    assert abs(float(fro) - np.linalg.norm(R)) <= 1e-12 * np.linalg.norm(R)
+    _, spec = rlu.reconstruct_error(*args, power_iters=300)
+    top = np.linalg.norm(R, 2)
+    assert top * 0.97 <= float(spec) <= top * (1 + 1e-12)
