@@ -1335,28 +1335,37 @@ int32_t launch_lu_reg_batched(bool crout, int rows_per_cta, const LuArgs* table_
   for (int g : {17, 18}) add(g);         // one CTA for small problems, several per SM
   const bool par = fork != nullptr && np > 1;
   if (par) RLU_CUDA_TRY(cudaEventRecord(fork->fork, s));
-  for (int i = 0; i < np; ++i) {
+  int32_t st = RLU_OK;
+  int used = 0;  // helper streams that wait for the fork
+  for (int i = 0; i < np && st == RLU_OK; ++i) {
     const Part& p = parts[i];
     cudaStream_t gs = s;
     if (par) {
       gs = fork->hs[i % kLuSide];
-      if (i < kLuSide) RLU_CUDA_TRY(cudaStreamWaitEvent(gs, fork->fork, 0));
+      if (i < kLuSide) {
+        if (cudaStreamWaitEvent(gs, fork->fork, 0) != cudaSuccess) {
+          st = RLU_ECUDA;
+          break;
+        }
+        ++used;
+      }
     }
     if (p.g == 17)
-      RLU_TRY(lu_batched_group<1>(crout, table_dev, p.first, p.count, 1, p.pw, gs));
+      st = lu_batched_group<1>(crout, table_dev, p.first, p.count, 1, p.pw, gs);
     else if (p.g == 18)
-      RLU_TRY(lu_batched_group<2>(crout, table_dev, p.first, p.count, 1, p.pw, gs));
+      st = lu_batched_group<2>(crout, table_dev, p.first, p.count, 1, p.pw, gs);
     else if (rows_per_cta == 512)
-      RLU_TRY(lu_batched_group<4>(crout, table_dev, p.first, p.count, p.g, p.pw, gs));
+      st = lu_batched_group<4>(crout, table_dev, p.first, p.count, p.g, p.pw, gs);
     else
-      RLU_TRY(lu_batched_group<2>(crout, table_dev, p.first, p.count, p.g, p.pw, gs));
+      st = lu_batched_group<2>(crout, table_dev, p.first, p.count, p.g, p.pw, gs);
   }
-  if (par)
-    for (int i = 0; i < np && i < kLuSide; ++i) {
-      RLU_CUDA_TRY(cudaEventRecord(fork->join[i], fork->hs[i]));
-      RLU_CUDA_TRY(cudaStreamWaitEvent(s, fork->join[i], 0));
-    }
-  return RLU_OK;
+  // joined also after an error: what follows on s comes after everything launched above
+  for (int i = 0; i < used; ++i) {
+    if (cudaEventRecord(fork->join[i], fork->hs[i]) != cudaSuccess ||
+        cudaStreamWaitEvent(s, fork->join[i], 0) != cudaSuccess)
+      st = st == RLU_OK ? (int32_t)RLU_ECUDA : st;
+  }
+  return st;
 }
 
 }  // namespace rlu
