@@ -51,18 +51,11 @@ struct Tables {
 
 constexpr int kSmallK = 64;
 
-// LU group of a problem with R rows (see rlu_batch) and its rows per CTA: small problems
-// take one narrow CTA, so that several of them share an SM.
-int lu_group(int64_t R, int rows_per_cta, int* rpc) {
-  if (R <= 128) {
-    *rpc = 128;
-    return 17;
-  }
-  if (R <= 256 && rows_per_cta == 512) {
-    *rpc = 256;
-    return 18;
-  }
-  *rpc = rows_per_cta;
+// LU group of a problem with R rows (see rlu_batch): small problems take one CTA of few rows, so
+// that several of them share an SM.
+int lu_group(int64_t R, int rows_per_cta) {
+  if (R <= 128) return 17;
+  if (R <= 256 && rows_per_cta == 512) return 18;
   return (int)ceil_div(R, rows_per_cta);
 }
 
@@ -172,7 +165,7 @@ struct rlu_batch {
   int64_t max_m = 0, max_n = 0;
   int max_k = 0, max_l = 0, max_kp = 0;
   // LU groups: 1..16 = clusters of that many CTAs of lu_rows_per_cta rows; 17 / 18 = one CTA
-  // of 128 / 256 threads for problems of at most 128 / 256 rows
+  // for problems of at most 128 / 256 rows (every CTA: 128 control and 128 update threads)
   int first_y[rlu::kLuGroups] = {}, count_y[rlu::kLuGroups] = {}, first_b[rlu::kLuGroups] = {},
       count_b[rlu::kLuGroups] = {}, wide_y[rlu::kLuGroups] = {}, wide_b[rlu::kLuGroups] = {};
   int launches = 0;
@@ -309,12 +302,12 @@ extern "C" int32_t rlu_batch_create(const rlu_problem* problems, int32_t count, 
     u.nonfinite = p.info ? &p.info->nonfinite : nullptr;
     u.status = p.info ? &p.info->status : nullptr;
     u.posg = pos; u.psg = ps; u.p0 = 0; u.pw = p.l; u.nb = kMaxL;
-    gy_of[(size_t)i] = lu_group(p.m, opt.lu_rows_per_cta, &u.rpc);
+    gy_of[(size_t)i] = lu_group(p.m, opt.lu_rows_per_cta);
     luy_all[(size_t)i] = u;
     u.X = Bb; u.ldx = L.ldb; u.R = (int)p.n; u.C = p.k; u.perm = p.Q;
     u.zero_step = p.info ? &p.info->first_zero_pivot_b : nullptr;
     u.pw = p.k;
-    gb_of[(size_t)i] = lu_group(p.n, opt.lu_rows_per_cta, &u.rpc);
+    gb_of[(size_t)i] = lu_group(p.n, opt.lu_rows_per_cta);
     lub_all[(size_t)i] = u;
     float* Lhi = mixed ? reinterpret_cast<float*>(ws + L.Lhi) : nullptr;
     float* Llo = mixed ? reinterpret_cast<float*>(ws + L.Llo) : nullptr;

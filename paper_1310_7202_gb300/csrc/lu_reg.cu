@@ -1173,8 +1173,7 @@ static int32_t trail(const LuArgs& in, T* X, int c_begin, int c_end, int p0, int
 template <typename T, bool CROUT, int RT, int NC, int pw_max, bool SOLO = false>
 static int32_t try_launch(const LuArgs& in, cudaStream_t s, bool* launched) {
   *launched = false;
-  const int rpc = NC * RT;
-  const int ncta = (int)ceil_div(in.R, rpc);
+  const int ncta = (int)ceil_div(in.R, NC * RT);
   if (ncta > (SOLO ? 1 : 16)) return RLU_OK;
   int dev = 0;
   RLU_CUDA_TRY(cudaGetDevice(&dev));
@@ -1216,7 +1215,6 @@ static int32_t try_launch(const LuArgs& in, cudaStream_t s, bool* launched) {
   // no position state or pivot-row buffer: the one-launch kernel takes the problem
   if (!in.posg || !in.psg || !in.u12) return RLU_OK;
   LuArgs a = in;
-  a.rpc = rpc;
   a.nb = pw;
   T* X = static_cast<T*>(in.X);
   T* U12 = static_cast<T*>(in.u12);
@@ -1240,7 +1238,11 @@ static int32_t try_launch(const LuArgs& in, cudaStream_t s, bool* launched) {
 
 template <typename T, bool CROUT>
 static int32_t launch_reg_t(const LuArgs& a, cudaStream_t s, bool* launched) {
-  // threads per CTA, rows per thread and panel columns by the number of rows
+  // threads per CTA, rows per thread and panel columns by the number of rows. The eight-row forms
+  // of 8-byte elements spill (1.2 to 1.4 KB a thread) and still win over the ones they replaced:
+  // FP64 factorizations of 20000 x 1000, k = 40, 6.6 -> 5.3 ms and 32768 x 600, k = 76, 14.0 ->
+  // 12.1; fast randomized LUs of 20000 x 1000, k = 40, 1.48 -> 1.40 ms and 30000 x 1024, k = 60,
+  // 1.80 -> 1.69.
   const int R = a.R;
   auto go = [&](int rows, auto f) -> int32_t {
     return (!*launched && R <= rows) ? f() : (int32_t)RLU_OK;
@@ -1277,15 +1279,15 @@ int32_t launch_lu_reg(int32_t dtype, bool crout, const LuArgs& a, cudaStream_t s
   return RLU_OK;
 }
 
-// Batched LUs of problems that fit one register panel (C <= NB - 1 = 76 FP32 columns, R <=
-// 16 x rows_per_cta): the table on the device is grouped by cluster size (ceil(R /
-// rows_per_cta) CTAs); group g starts at table entry first[g] and holds count[g] problems.
-// rows_per_cta is 512 or 256 (twice as many CTAs per problem). A panel of 76 columns of 512 rows
-// takes more than half an SM's shared memory, and a step of one CTA leaves its SM idle while it
-// waits; the groups of 512-row CTAs are therefore launched in two parts, up to 48 columns (108 KB
-// a CTA) and more, and no CTA takes more than 128 registers a thread, so that two share an SM.
-// With the longest LUs of a group first, 512 problems (m <= 2048, k <= 64) 1239 -> 1168 us, of
-// which 16 us are the order of the C product's tiles.
+// Batched LUs of problems that fit one panel (C <= 76 FP32 columns, R <= 16 x rows_per_cta): the
+// table on the device is grouped by cluster size (ceil(R / rows_per_cta) CTAs); group g starts at
+// table entry first[g] and holds count[g] problems. rows_per_cta is 512 or 256 (twice as many
+// CTAs per problem). A panel of 76 columns of 512 rows takes more than half an SM's shared
+// memory, and a step of one CTA leaves its SM idle while it waits; the groups of 512-row CTAs are
+// therefore launched in two parts, up to 48 columns (108 KB a CTA) and more, and no CTA takes
+// more than 128 registers a thread, so that two share an SM. With the longest LUs of a group
+// first, 512 problems (m <= 2048, k <= 64) 1239 -> 1168 us, of which 16 us are the order of the C
+// product's tiles.
 template <int RT>
 static int32_t lu_batched_group(bool crout, const LuArgs* table_dev, int first, int count, int g,
                                 int pw, cudaStream_t s) {

@@ -10,7 +10,7 @@ struct LuArgs {
   int64_t ldx;         // >= R
   int R, C;            // rows, steps (C <= R)
   int nb;              // panel width (set by the launcher)
-  int rpc;             // rows per CTA (set by the launcher)
+  int rpc;             // rows per CTA (set by the launcher; one-launch kernel only)
   int32_t* perm;       // [R] out: row at final position p
   int32_t* zero_step;  // out: first step with a zero pivot, -1 if none (may be NULL)
   int32_t* nonfinite;  // out: OR-ed with 1 when a NaN/Inf is met (may be NULL)
@@ -42,8 +42,8 @@ int32_t launch_lu_reg(int32_t dtype, bool crout, const LuArgs& a, cudaStream_t s
 // each; the device table is grouped (entries first[g] .. first[g] + count[g] - 1; first and
 // count are host arrays of kLuGroups entries): g = 1..16 is the cluster size ceil(R /
 // rows_per_cta), g = 17 one CTA for R <= 128, g = 18 one CTA for R <= 256; every CTA has 128
-// control and 128 update threads. Each entry carries its rpc (rows per CTA), p0 = 0, pw = C and
-// its own position state (posg, psg).
+// control and 128 update threads. Each entry carries p0 = 0, pw = C and its own position state
+// (posg, psg).
 static constexpr int kLuGroups = 19;
 // Helper streams for the groups: with fork != nullptr every non-empty group is launched on
 // its own helper stream (fork / join events around them on s), so that the groups' CTAs
