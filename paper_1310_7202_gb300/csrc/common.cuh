@@ -42,9 +42,9 @@ int sm_count();
 
 // Lets a kernel be launched with as much dynamic shared memory as the device has for a CTA beside
 // the kernel's static part. The limit belongs to the function and is shared by all host threads,
-// so it is set once per device and to the largest value: set to each call's size before its
-// launch, a thread with a smaller one makes another's launch fail. What a launch takes, and so
-// how many CTAs share an SM, is its own size.
+// so every call sets it to the same, largest value: set to each call's size before its launch, a
+// thread with a smaller one makes another's launch fail. What a launch takes, and so how many
+// CTAs share an SM, is its own size.
 int32_t allow_smem_of(const void* kernel);
 template <typename F>
 int32_t allow_smem(F* kernel) {

@@ -13,7 +13,6 @@
 #include <atomic>
 #include <map>
 #include <mutex>
-#include <set>
 #include <utility>
 
 #include "common.cuh"
@@ -59,17 +58,23 @@ int sm_count() {
 
 int32_t allow_smem_of(const void* kernel) {
   static std::mutex mu;
-  static std::set<std::pair<int, const void*>> done;
-  int dev = 0, optin = 0;
+  static std::map<std::pair<int, const void*>, int> limits;  // the code's and the device's, for good
+  int dev = 0, optin = 0, limit = 0;
   RLU_CUDA_TRY(cudaGetDevice(&dev));
-  std::lock_guard<std::mutex> lock(mu);
-  if (done.count({dev, kernel})) return RLU_OK;
-  cudaFuncAttributes at{};
-  RLU_CUDA_TRY(cudaFuncGetAttributes(&at, kernel));
-  RLU_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  RLU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    optin - (int)at.sharedSizeBytes));
-  done.insert({dev, kernel});
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    const auto at = limits.find({dev, kernel});
+    if (at != limits.end()) {
+      limit = at->second;
+    } else {
+      cudaFuncAttributes fa{};
+      RLU_CUDA_TRY(cudaFuncGetAttributes(&fa, kernel));
+      RLU_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+      limits[{dev, kernel}] = limit = optin - (int)fa.sharedSizeBytes;
+    }
+  }
+  // set each time: a device reset forgets it
+  RLU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
   return RLU_OK;
 }
 
