@@ -99,16 +99,26 @@ __global__ void __launch_bounds__(256) k_range(ResidualArgs a, int lu_exp, int t
   scan(static_cast<const TA*>(a.A), a.m, a.n, a.lda, big[0]);
   scan(static_cast<const TLU*>(a.L), a.k, a.m, a.ldl, big[1]);
   scan(static_cast<const TLU*>(a.U), a.k, a.n, a.ldu, big[2]);
+  __shared__ uint32_t red[3][8];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     const uint32_t w = __reduce_max_sync(0xffffffffu, big[i]);
-    if ((threadIdx.x & 31) == 0 && w) atomicMax(mx + i, w);
+    if ((threadIdx.x & 31) == 0) red[i][threadIdx.x >> 5] = w;
   }
-  __threadfence();
   __syncthreads();
+  if (threadIdx.x >= 32) return;
+  if (threadIdx.x < 3) {  // one atomic a block; one a warp cost more than the count below
+    uint32_t w = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) w = max(w, red[threadIdx.x][q]);
+    atomicMax(mx + threadIdx.x, w);
+    __threadfence();
+  }
+  __syncwarp();
   if (threadIdx.x == 0 && atomicAdd(mx + 3, 1u) == gridDim.x - 1) {  // the last block
     __threadfence();
     int e[3];
+#pragma unroll
     for (int i = 0; i < 3; ++i) e[i] = (int)(__ldcg(mx + i) >> 23);
     if (e[0] + max(e[0], e[1] + e[2] + lu_exp) > top_exp) mx[0] = 0;
   }
